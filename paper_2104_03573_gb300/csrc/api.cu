@@ -427,7 +427,6 @@ struct SteadyWs {
   uint64_t* offs;
   char* zero_begin;
   double* cellP;
-  double* cellD;
   double* qbin;
   long long* cellPq;
   long long* cellDq;
@@ -495,7 +494,6 @@ SteadyWs layout_steady(char* base, int G, int n, int nc, uint64_t total, bool gr
   c.off = (c.off + 255) & ~(size_t)255;
   w.zero_begin = base ? base + c.off : nullptr;
   w.cellP = nc > 0 ? c.take<double>((size_t)G * nc * 4) : nullptr;
-  w.cellD = nc > 0 ? c.take<double>((size_t)G * (nc + 1) * 4) : nullptr;
   w.qbin = c.take<double>((size_t)G * n);
   w.cellPq = nc > 0 ? c.take<long long>((size_t)G * nc * 4) : nullptr;
   w.cellDq = nc > 0 ? c.take<long long>((size_t)G * (nc + 1) * 4) : nullptr;
@@ -689,7 +687,7 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
   C.refill_min = p->refill_threshold;
   C.tail_max = p->tail_lanes == 0 ? 8 : (p->tail_lanes < 0 ? 0 : p->tail_lanes);
   C.fused = fused ? 1 : 0;
-  C.take_chunk = G > 1 ? 1024u : 256u;
+  C.take_chunk = G > 1 ? 1024u : 256u;   // at most: a warp of a batch stays on one geometry longer
   C.cell_flux_axis = p->cell_flux_axis ? 1 : 0;
   C.ext = (p->n_regions > 0 || nscat > 0) ? 1 : 0;
   for (int g = 0; g < G; ++g) C.ext |= uses_ext(m, geoms[g]->host) ? 1 : 0;
@@ -712,7 +710,6 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
   }
   Acc A{};
   A.cellP = w.cellP;
-  A.cellD = w.cellD;
   A.qbin = w.qbin;
   A.cellPq = w.cellPq;
   A.cellDq = w.cellDq;

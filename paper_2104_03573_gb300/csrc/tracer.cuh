@@ -68,9 +68,8 @@ struct RunCfg {
   int tail_max;         // FP32 steady tracer: the tail's draw slots serve warps with at most
                         // this many particles in flight once the work counter has run out (0: off)
   int fused;            // FP32 gradient: the forward tallies and the gradient in one pass
-  // particle indices a warp takes from the work counter at once (WarpRun):
-  // 1024 for a batch of geometries (a warp stays on one geometry longer),
-  // 256 otherwise (a shorter drain); 0 counts as 32
+  // particle indices a warp takes at once (WarpRun), a multiple of 32; set by
+  // take_chunk() at the launch from the most a warp takes
   unsigned take_chunk;
 };
 
@@ -168,11 +167,10 @@ constexpr int kSumCopies = 64;
 constexpr int kGradStride = 4 + 2 * kMaxDirs;
 
 struct Acc {
-  double* cellP;              // [G][nc][4]   per-cell direct / partial-cell sums (FP64 path)
-  double* cellD;              // [G][nc+1][4] difference array of full-cell sums (FP64 path)
+  double* cellP;              // [G][nc][4]   per-cell sums (FP64 path)
   double* qbin;               // [G][n_bins]  (FP64 path)
-  long long* cellPq;          // [G][nc][4]   fixed-point counterparts (FP32 path)
-  long long* cellDq;          // [G][nc+1][4]
+  long long* cellPq;          // [G][nc][4]   fixed-point partial-cell sums (FP32 path)
+  long long* cellDq;          // [G][nc+1][4] difference array of its full-cell sums
   long long* qbinq;           // [G][n_bins]
   double* dsc;                // [G][8] (transient: [kSumCopies][8]): sumX, sumX2, signed emitted,
                               // signed absorbed, -, -, -, absorbed
@@ -964,19 +962,34 @@ struct GradReplay {
   __device__ __forceinline__ double spec_term(double) const { return (double)pd; }
 };
 
-// A warp's run of particle indices [cb, ce), taken from the run's work
-// counter `chunk` at a time (RunCfg::take_chunk): one returning atomic on
-// that single address per chunk instead of one per warp refill.  take()
-// (called by the whole warp) returns this lane's index among the lanes in
-// `need` (the others' values are meaningless) and checks the time budget at
-// every take of the counter (particles shorter than the per-event check
-// interval would otherwise never look).  dry: the counter has run out; with
-// cb >= ce the warp has nothing left to hand out.
+// A warp's run of particle indices [cb, ce).  The first `chunk` indices are
+// the warp's by its number in the grid (start), later ones come from the
+// run's work counter, `chunk` at a time: one returning atomic on that single
+// address per chunk instead of one per warp refill, and none where the grid
+// holds the whole run.  take() (called by the whole warp) returns this lane's
+// index among the lanes in `need` (the others' values are meaningless).  The
+// time budget is checked at the start and at every take of the counter
+// (particles shorter than the per-event check interval would otherwise never
+// look).  dry: the counter has run out; with cb >= ce the warp has nothing
+// left to hand out.
 struct WarpRun {
   uint64_t cb = 0, ce = 0;
+  uint64_t base = 0;   // indices the grid's warps hold from the start
+  unsigned chunk = 32u;
   bool dry = false;
+
+  // Warps are numbered block by block across the grid (warp 0 of every block
+  // first), so a run with fewer chunks than warps spreads over all SMs.
+  __device__ __forceinline__ void start(unsigned chunk_, uint64_t total, uint64_t deadline, int* flags) {
+    chunk = chunk_;
+    base = (uint64_t)gridDim.x * (blockDim.x >> 5) * chunk;
+    cb = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * chunk;
+    ce = cb + chunk < total ? cb + chunk : total;
+    dry = base >= total;
+    if ((threadIdx.x & 31u) == 0u && globaltimer_ns() > deadline) atomicOr(flags, 1);
+  }
   __device__ __forceinline__ uint64_t take(unsigned need, unsigned lane, unsigned long long* work, uint64_t total,
-                                           unsigned chunk, uint64_t deadline, int* flags) {
+                                           uint64_t deadline, int* flags) {
     const unsigned cnt = __popc(need);
     const unsigned rank = __popc(need & ((1u << lane) - 1u));
     const uint64_t left = cb < ce ? ce - cb : 0;
@@ -985,13 +998,14 @@ struct WarpRun {
       cb += cnt;
       return k;
     }
-    chunk = chunk < 32u ? 32u : chunk;   // at least a warp's refill
-    unsigned long long nb = 0;
-    if (lane == 0) {
-      nb = atomicAdd(work, (unsigned long long)chunk);
-      if (globaltimer_ns() > deadline) atomicOr(flags, 1);
+    unsigned long long nb = total;
+    if (!dry) {
+      if (lane == 0) {
+        nb = base + atomicAdd(work, (unsigned long long)chunk);
+        if (globaltimer_ns() > deadline) atomicOr(flags, 1);
+      }
+      nb = __shfl_sync(0xffffffffu, nb, 0);
     }
-    nb = __shfl_sync(0xffffffffu, nb, 0);
     const uint64_t k = rank < left ? cb + rank : nb + (rank - left);
     cb = nb + (cnt - left);
     ce = nb + chunk < total ? nb + chunk : total;

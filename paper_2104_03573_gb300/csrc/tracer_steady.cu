@@ -203,6 +203,69 @@ struct ThreadAcct {
   }
 };
 
+// A block's book-keeping (shared memory), for runs of one geometry.  Every
+// lane of the grid flushing its own fields queued 8e5 atomics on seven
+// addresses (about 0.4 ms, whatever the run's length: a gray slab of 1e5
+// particles 502 us, 35 us without them); a warp's lanes are summed by
+// shuffles, the block's warps here, and a block adds once.
+struct BlockAcct {
+  unsigned long long ev, trunc, maxev, traced;
+  long long sxq, s_emit, s_abs, absorbed;
+  double sx2;
+
+  __device__ __forceinline__ void reset() {
+    ev = trunc = maxev = traced = 0ull;
+    sxq = s_emit = s_abs = absorbed = 0;
+    sx2 = 0.0;
+  }
+  // called by all 32 lanes of a warp
+  __device__ __forceinline__ void add(const ThreadAcct& t) {
+    constexpr unsigned kAll = 0xffffffffu;
+    unsigned long long ev_w = t.ev, sx_w = (unsigned long long)t.sxq;
+    long long se = t.s_emit, sa = t.s_abs;
+    double s2 = t.sx2;
+    unsigned long long tr = t.traced;
+    const unsigned tc = __reduce_add_sync(kAll, t.trunc), ab = __reduce_add_sync(kAll, t.absorbed);
+    const unsigned mx = __reduce_max_sync(kAll, t.maxev);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      ev_w += __shfl_xor_sync(kAll, ev_w, o);
+      sx_w += __shfl_xor_sync(kAll, sx_w, o);
+      se += __shfl_xor_sync(kAll, se, o);
+      sa += __shfl_xor_sync(kAll, sa, o);
+      s2 += __shfl_xor_sync(kAll, s2, o);
+      tr += __shfl_xor_sync(kAll, tr, o);
+    }
+    if ((threadIdx.x & 31u) != 0u || tr == 0ull) return;
+    atomicAdd(&ev, ev_w);
+    if (tc) atomicAdd(&trunc, (unsigned long long)tc);
+    atomicMax(&maxev, (unsigned long long)mx);
+    atomicAdd(&traced, tr);
+    red_s64(&sxq, (long long)sx_w);
+    atomicAdd(&sx2, s2);
+    red_s64(&s_emit, se);
+    if (ab) {
+      red_s64(&s_abs, sa);
+      red_s64(&absorbed, (long long)ab);
+    }
+  }
+  // by one thread, after the block's warps have added
+  __device__ __forceinline__ void flush(const Acc& A) const {
+    if (traced == 0ull) return;
+    atomicAdd(&A.cnt[0], ev);
+    if (trunc) atomicAdd(&A.cnt[1], trunc);
+    atomicMax(&A.cnt[2], maxev);
+    atomicAdd(&A.cnt[3], traced);
+    atomicAdd(&A.dsc[0], (double)sxq * kFxInv);
+    atomicAdd(&A.dsc[1], sx2);
+    atomicAdd(&A.dsc[2], (double)s_emit);
+    if (absorbed) {
+      atomicAdd(&A.dsc[3], (double)s_abs);
+      atomicAdd(&A.dsc[7], (double)absorbed);
+    }
+  }
+};
+
 // Gradient pass: the open period closes at the particle's end (X = X_f; a
 // fused pass adds its listed periods' a X_f too), then the resampling and
 // specularity terms and the directional values.
@@ -640,6 +703,8 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
     s_cD = s_cP + (size_t)nc * 4;
     for (int i = threadIdx.x; i < nc * 4 + (nc + 1) * 4; i += blockDim.x) s_cP[i] = 0;
   }
+  __shared__ BlockAcct s_acct;
+  if (threadIdx.x == 0) s_acct.reset();
   __syncthreads();
 
   const unsigned lane = threadIdx.x & 31u;
@@ -688,6 +753,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   const uint64_t n_parked = TK ? min(*(volatile unsigned long long*)A.park_n, (unsigned long long)A.park_cap) : 0;
   bool pool_dry = false;   // the same in every lane: nothing left to hand out
   WarpRun run;              // main kernel: the warp's particle indices not yet handed out
+  if constexpr (!TK) run.start(C.take_chunk, C.total, deadline, A.flags);
   // the tallies of the lane's geometry
   auto bind = [&](int g) {
     if (g != acct.g) {
@@ -793,7 +859,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
           if (base + cnt >= avail) pool_dry = true;
           k = base + rank;
         } else {
-          k = run.take(need, lane, A.work, C.total, C.take_chunk, deadline, A.flags);
+          k = run.take(need, lane, A.work, C.total, deadline, A.flags);
           avail = C.total;
           if (run.empty()) pool_dry = true;
         }
@@ -898,8 +964,13 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
     alive = false;
     drained = pool_dry;
   }
-  if (!GRAD || C.fused) acct.flush(A);
+  const bool one_geom = C.n_geoms == 1;
+  if (!GRAD || C.fused) {
+    if (one_geom) s_acct.add(acct);
+    else acct.flush(A);
+  }
   __syncthreads();
+  if (threadIdx.x == 0 && one_geom) s_acct.flush(A);
   if (S.qbin_in_smem) {
     for (int i = threadIdx.x; i < n; i += blockDim.x)
       if (s_qbin[i] != 0) atomicAdd(reinterpret_cast<unsigned long long*>(&A.qbinq[i]), (unsigned long long)s_qbin[i]);
@@ -932,26 +1003,36 @@ __global__ void k_finalize_steady(const GeoRun* geos, MatView M, RunCfg C, Acc A
   const double N = (double)G.n_norm;
   const double E_eff = G.E_tot / N;
   const double C_tot = M.sums[0];
-  if (nc > 0 && threadIdx.x == 0) {
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (nc > 0 && warp < 4) {
+    // cells: warp b takes component b (T, q_x, q_y, q_z) of all cells, the
+    // difference array folded by a warp scan of the integer sums, 32 cells at
+    // a time (one thread over all cells and components took 68 us for 50
+    // cells, all of it load latency; the kernel now takes 6 us)
+    const int b = (int)warp;
     const double Vc = G.V_box / (double)nc;
-    const double kT = E_eff / (C_tot * Vc);
-    const double kq = E_eff / Vc;
-    double run[4] = {0.0, 0.0, 0.0, 0.0};
+    const double k = b == 0 ? E_eff / (C_tot * Vc) : E_eff / Vc;
     const double* P = A.cellP + (size_t)g * nc * 4;
-    const double* D = A.cellD + (size_t)g * (nc + 1) * 4;
     const long long* Pq = A.cellPq + (size_t)g * nc * 4;
     const long long* Dq = A.cellDq + (size_t)g * (nc + 1) * 4;
-    long long runq[4] = {0, 0, 0, 0};
-    for (int c = 0; c < nc; ++c) {
-      double v[4];
-      for (int b = 0; b < 4; ++b) {
-        run[b] += D[c * 4 + b];
-        runq[b] += Dq[c * 4 + b];
-        v[b] = P[c * 4 + b] + run[b] + (double)(Pq[c * 4 + b] + runq[b]) * kFxInv;
+    long long carry = 0;
+    for (int c0 = 0; c0 < nc; c0 += 32) {
+      const int c = c0 + (int)lane;
+      const bool in = c < nc;
+      long long run = in ? Dq[c * 4 + b] : 0;
+      const long long pq = in ? Pq[c * 4 + b] : 0;
+      const double pd = in ? P[c * 4 + b] : 0.0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, run, o);
+        if ((int)lane >= o) run += y;
       }
-      if (O.T) O.T[(size_t)g * nc + c] = (kT * v[0]) * 1e-12;
-      if (O.q)
-        for (int b = 0; b < 3; ++b) O.q[((size_t)g * nc + c) * 3 + b] = (kq * v[1 + b]) * 1e-9;
+      run += carry;
+      carry = __shfl_sync(0xffffffffu, run, 31);
+      const double v = pd + (double)(pq + run) * kFxInv;
+      if (!in) continue;
+      if (b == 0 && O.T) O.T[(size_t)g * nc + c] = (k * v) * 1e-12;
+      if (b > 0 && O.q) O.q[((size_t)g * nc + c) * 3 + (b - 1)] = (k * v) * 1e-9;
     }
   }
   if (O.det && C.n_regs > 0) {
@@ -1010,7 +1091,7 @@ __global__ void k_finalize_steady(const GeoRun* geos, MatView M, RunCfg C, Acc A
       O.q_bin[j] = (kb * (A.qbin[j] + (double)A.qbinq[j] * kFxInv)) * 1e-9;
     }
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 128) {   // (a warp the cells leave free)
     const double sx = A.dsc[g * 8 + 0], sx2 = A.dsc[g * 8 + 1];
     const double nt = (double)A.cnt[g * 4 + 3];
     const double mean = sx / nt;
@@ -1101,7 +1182,9 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   const int b = (bps > 0 && bps < occ) ? bps : occ;
-  kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, offs, M, C, A, S);
+  RunCfg R = C;
+  R.take_chunk = take_chunk(C.total, (uint64_t)sm_count() * b * (TPB / 32), C.take_chunk);
+  kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, offs, M, R, A, S);
   return cudaGetLastError();
 }
 

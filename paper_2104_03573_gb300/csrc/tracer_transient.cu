@@ -46,6 +46,48 @@ __device__ __forceinline__ void transient_finish(const Particle<R>& p, int out, 
   if (A.events_pp) A.events_pp[idx] = (uint32_t)nev;
 }
 
+// The run counters of a warp's finished particles, spread over its lanes:
+// lane 0 events, 1 truncated, 2 most events, 3 traced, 4 sum of signs emitted,
+// 5 sum of signs absorbed, 6 absorbed.  One register pair a lane, and one
+// atomic per counter and warp at the kernel's end, where each particle added
+// five to six to a few addresses (a wall pulse of 2e5 particles: 1.2e6
+// atomics, two thirds of its kernel).
+struct WarpAcct {
+  unsigned long long v = 0ull;
+  // called by all 32 lanes; `ended`: this lane's particle ended with `out`
+  __device__ __forceinline__ void add(bool ended, int out, uint32_t e, float s, unsigned lane) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const unsigned m = __ballot_sync(kAll, ended);
+    if (!m) return;
+    const unsigned mp = __ballot_sync(kAll, ended && s > 0.0f);
+    const unsigned ma = __ballot_sync(kAll, ended && out == STEP_ABSORBED);
+    const unsigned mt = __ballot_sync(kAll, ended && out == STEP_TRUNCATED);
+    const unsigned nev = ended ? e + 1u : 0u;
+    const unsigned lo = __reduce_add_sync(kAll, nev & 0xffffu), hi = __reduce_add_sync(kAll, nev >> 16);
+    const unsigned mx = __reduce_max_sync(kAll, nev);
+    const unsigned long long ev = ((unsigned long long)hi << 16) + lo;
+    const long long se = 2ll * __popc(mp) - __popc(m), sa = 2ll * __popc(mp & ma) - __popc(ma);
+    if (lane == 2) {
+      v = mx > v ? mx : v;
+    } else {
+      v += lane == 0   ? ev
+           : lane == 1 ? (unsigned long long)__popc(mt)
+           : lane == 3 ? (unsigned long long)__popc(m)
+           : lane == 4 ? (unsigned long long)se
+           : lane == 5 ? (unsigned long long)sa
+                       : (unsigned long long)__popc(ma);
+    }
+  }
+  __device__ __forceinline__ void flush(unsigned lane, const Acc& A) const {
+    unsigned long long* cnt = A.cnt + sum_copy() * 4;
+    double* dsc = A.dsc + sum_copy() * 8;
+    if (v == 0ull || lane > 6) return;
+    if (lane == 2) atomicMax(cnt + 2, v);
+    else if (lane < 4) atomicAdd(cnt + lane, v);
+    else atomicAdd(dsc + (lane == 4 ? 2 : (lane == 5 ? 3 : 7)), (double)(long long)v);
+  }
+};
+
 #if MCBTE_F64
 __global__ void __launch_bounds__(256) k_transient_fp64(const GeoRun* __restrict__ geos, MatView M, RunCfg C, Acc A) {
   const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -283,7 +325,11 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
   const unsigned lane = threadIdx.x & 31u;
   const uint2 key = run_key(C);
   WarpRun run;   // the warp's particle indices not yet handed out
+  run.start(C.take_chunk, C.total, deadline, A.flags);
   Particle<float> p;
+  p.e = 0u;
+  p.s = 0.0f;
+  WarpAcct acct;
   bool alive = false;
   bool drained = false;   // as in the steady tracer: idle lanes stay until the warp is drained
   uint64_t idx = 0;
@@ -297,7 +343,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
       if (__all_sync(kAll, drained)) break;
       const unsigned need = __ballot_sync(kAll, !alive && !drained);
       if (need) {
-        const uint64_t k = run.take(need, lane, A.work, C.total, C.take_chunk, deadline, A.flags);
+        const uint64_t k = run.take(need, lane, A.work, C.total, deadline, A.flags);
         if (!alive && !drained) {
           idx = k;
           if (idx >= C.total || (*(volatile int*)A.flags & 1)) {
@@ -358,34 +404,39 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
       }
       if constexpr (TAVG) warp_bin_averages(k, t_end, p, tmeas, C, A.snap);
       else warp_snapshots(k, p, tmeas, cinv, C, A.snap);
-      if (!alive) continue;
-      if (out == STEP_ALIVE) {
-        if constexpr (TAVG) p.mi = mi_next;
-        else p.mi += k;
-        p.t = t_end;
+      bool ended = false;
+      if (alive) {
+        if (out == STEP_ALIVE) {
+          if constexpr (TAVG) p.mi = mi_next;
+          else p.mi += k;
+          p.t = t_end;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) p.x[a] = p.x[a] + seg * p.u[a];
-        if (fin) {
-          out = STEP_DONE;
-        } else {
-          GradOff off;
-          out = apply_event<float, GradOff, TallyNone, EXT>(p, G, M, relax, binf, C, key.x, key.y, rlx, rlx2, face, seg,
-                                                            TallyNone(), off, 0.0);
+          for (int a = 0; a < 3; ++a) p.x[a] = p.x[a] + seg * p.u[a];
+          if (fin) {
+            out = STEP_DONE;
+          } else {
+            GradOff off;
+            out = apply_event<float, GradOff, TallyNone, EXT>(p, G, M, relax, binf, C, key.x, key.y, rlx, rlx2, face, seg,
+                                                              TallyNone(), off, 0.0);
+          }
+        }
+        if (out == STEP_ALIVE && (p.e & 255u) == 0u && globaltimer_ns() > deadline) {
+          atomicOr(A.flags, 1);
+          out = STEP_TRUNCATED;
+        }
+        if (out != STEP_ALIVE) {
+          ended = true;
+          alive = false;
+          if (A.events_pp) A.events_pp[idx] = p.e + 1u;
+          if (!C.win_last) mark_done(A.tstate, idx);
+        } else if (!C.win_last && p.mi >= C.win_end) {
+          save_state(A.tstate, idx, p);
+          alive = false;
         }
       }
-      if (out == STEP_ALIVE && (p.e & 255u) == 0u && globaltimer_ns() > deadline) {
-        atomicOr(A.flags, 1);
-        out = STEP_TRUNCATED;
-      }
-      if (out != STEP_ALIVE) {
-        transient_finish(p, out, idx, A);
-        if (!C.win_last) mark_done(A.tstate, idx);
-        alive = false;
-      } else if (!C.win_last && p.mi >= C.win_end) {
-        save_state(A.tstate, idx, p);
-        alive = false;
-      }
+      acct.add(ended, out, p.e, p.s, lane);
     }
+    acct.flush(lane, A);
     return;
   }
   // snapshots into detector regions: the per-lane loop
@@ -394,44 +445,45 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
       if (__all_sync(kAll, drained)) break;
       const unsigned need = __ballot_sync(kAll, !alive && !drained);
       if (need) {
-        const uint64_t k = run.take(need, lane, A.work, C.total, C.take_chunk, deadline, A.flags);
+        const uint64_t k = run.take(need, lane, A.work, C.total, deadline, A.flags);
         if (!alive && !drained) {
           idx = k;
           if (idx >= C.total || (*(volatile int*)A.flags & 1)) {
             drained = true;
-            continue;
-          }
-          if (C.win_first) {
+          } else if (C.win_first) {
             p.pid = (uint32_t)idx;
             p.g = 0;
             emit<float, EXT>(p, G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, true, (float)C.t_max_ps);
             transient_start(p, C);
-            if (!C.win_last && p.mi >= C.win_end) {   // emitted after this window's last snapshot
-              save_state(A.tstate, idx, p);
-              continue;
-            }
-          } else if (!load_state(A.tstate, idx, p, M, binf, C)) {
-            continue;
+            if (!C.win_last && p.mi >= C.win_end) save_state(A.tstate, idx, p);   // emitted after this window
+            else alive = true;
+          } else if (load_state(A.tstate, idx, p, M, binf, C)) {
+            alive = true;
           }
-          alive = true;
         }
       }
-      if (!alive) continue;
-      int out = step_transient<float, EXT>(p, G, M, relax, binf, C, key.x, key.y, A.snap, tmeas, cinv);
-      if (out == STEP_ALIVE && (p.e & 255u) == 0u && globaltimer_ns() > deadline) {
-        atomicOr(A.flags, 1);
-        out = STEP_TRUNCATED;
+      int out = STEP_ALIVE;
+      bool ended = false;
+      if (alive) {
+        out = step_transient<float, EXT>(p, G, M, relax, binf, C, key.x, key.y, A.snap, tmeas, cinv);
+        if (out == STEP_ALIVE && (p.e & 255u) == 0u && globaltimer_ns() > deadline) {
+          atomicOr(A.flags, 1);
+          out = STEP_TRUNCATED;
+        }
+        if (out != STEP_ALIVE) {
+          ended = true;
+          alive = false;
+          if (A.events_pp) A.events_pp[idx] = p.e + 1u;
+          if (!C.win_last) mark_done(A.tstate, idx);
+        } else if (!C.win_last && p.mi >= C.win_end) {
+          // this window's snapshots are taken: park the particle at its event
+          save_state(A.tstate, idx, p);
+          alive = false;
+        }
       }
-      if (out != STEP_ALIVE) {
-        transient_finish(p, out, idx, A);
-        if (!C.win_last) mark_done(A.tstate, idx);
-        alive = false;
-      } else if (!C.win_last && p.mi >= C.win_end) {
-        // this window's snapshots are taken: park the particle at its event
-        save_state(A.tstate, idx, p);
-        alive = false;
-      }
+      acct.add(ended, out, p.e, p.s, lane);
     }
+    acct.flush(lane, A);
   }
 }
 
@@ -476,28 +528,43 @@ __global__ void k_finalize_transient(const GeoRun* geos, MatView M, RunCfg C, Ac
     o[2] = (kq * a2) * 1e3;
     o[3] = (kq * a3) * 1e3;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    // fold the copies of the run counters
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) {
+    // fold the copies of the run counters: a lane per copy, then a warp sum
+    // (whole numbers, so the order changes nothing)
+    const unsigned lane = threadIdx.x;
     unsigned long long c[4] = {0ull, 0ull, 0ull, 0ull};
-    double d[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int r = 0; r < kSumCopies; ++r) {
+    double d[3] = {0.0, 0.0, 0.0};
+    for (int r = (int)lane; r < kSumCopies; r += 32) {
       c[0] += A.cnt[r * 4 + 0];
       c[1] += A.cnt[r * 4 + 1];
       c[2] = c[2] > A.cnt[r * 4 + 2] ? c[2] : A.cnt[r * 4 + 2];
       c[3] += A.cnt[r * 4 + 3];
-      for (int k = 0; k < 8; ++k) d[k] += A.dsc[r * 8 + k];
+      d[0] += A.dsc[r * 8 + 2];
+      d[1] += A.dsc[r * 8 + 3];
+      d[2] += A.dsc[r * 8 + 7];
     }
-    for (int k = 0; k < MCBTE_NSTATS; ++k) stats[k] = 0.0;
-    stats[MCBTE_STAT_EVENTS] = (double)c[0];
-    stats[MCBTE_STAT_TRUNCATED] = (double)c[1];
-    stats[MCBTE_STAT_MAX_EVENTS] = (double)c[2];
-    stats[MCBTE_STAT_N] = (double)c[3];
-    stats[MCBTE_STAT_E_TOT] = G.E_tot;
-    stats[MCBTE_STAT_SIGNED_EMITTED] = d[2];
-    stats[MCBTE_STAT_SIGNED_ABSORBED] = d[3];
-    stats[MCBTE_STAT_ABSORBED] = d[7];
-    stats[MCBTE_STAT_STATUS] = (A.flags[0] & 1) ? (double)MCBTE_ERR_TIMEOUT
-                                                : (c[1] ? (double)MCBTE_WARN_TRUNCATED : 0.0);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      c[0] += __shfl_xor_sync(0xffffffffu, c[0], o);
+      c[1] += __shfl_xor_sync(0xffffffffu, c[1], o);
+      const unsigned long long m = __shfl_xor_sync(0xffffffffu, c[2], o);
+      c[2] = c[2] > m ? c[2] : m;
+      c[3] += __shfl_xor_sync(0xffffffffu, c[3], o);
+      for (int k = 0; k < 3; ++k) d[k] += __shfl_xor_sync(0xffffffffu, d[k], o);
+    }
+    if (lane == 0) {
+      for (int k = 0; k < MCBTE_NSTATS; ++k) stats[k] = 0.0;
+      stats[MCBTE_STAT_EVENTS] = (double)c[0];
+      stats[MCBTE_STAT_TRUNCATED] = (double)c[1];
+      stats[MCBTE_STAT_MAX_EVENTS] = (double)c[2];
+      stats[MCBTE_STAT_N] = (double)c[3];
+      stats[MCBTE_STAT_E_TOT] = G.E_tot;
+      stats[MCBTE_STAT_SIGNED_EMITTED] = d[0];
+      stats[MCBTE_STAT_SIGNED_ABSORBED] = d[1];
+      stats[MCBTE_STAT_ABSORBED] = d[2];
+      stats[MCBTE_STAT_STATUS] = (A.flags[0] & 1) ? (double)MCBTE_ERR_TIMEOUT
+                                                  : (c[1] ? (double)MCBTE_WARN_TRUNCATED : 0.0);
+    }
   }
 }
 
@@ -532,7 +599,9 @@ cudaError_t launch_transient_tav(const GeoRun* geos, const MatView& M, const Run
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   const int b = (bps > 0 && bps < occ) ? bps : occ;
-  kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, M, C, A, S);
+  RunCfg R = C;
+  R.take_chunk = take_chunk(C.total, (uint64_t)sm_count() * b * (TPB / 32), C.take_chunk);
+  kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, M, R, A, S);
   return cudaGetLastError();
 }
 template <int TPB, bool EXT>
