@@ -865,10 +865,6 @@ struct TransientWs {
   size_t bytes;
 };
 
-// FP32 transient time windows: measurement times per window.  Automatic
-// choice: the largest window whose [times][cells][4] x 8-byte slice of the
-// snapshot tally fits a third of the L2, so the snapshot atomics of a window
-// hit in L2 instead of read-modify-writing HBM.
 uint64_t transient_detectors(const mcbte_transient_params* p) {
   if (p->n_regions == 0) return (uint64_t)p->grid[0] * p->grid[1] * p->grid[2];
   uint64_t nd = 0;
@@ -877,9 +873,17 @@ uint64_t transient_detectors(const mcbte_transient_params* p) {
   return nd;
 }
 
+// FP32 transient time windows: measurement times per window.  Automatic
+// choice: the whole run for snapshots on the box grid, whose reductions add
+// whole 32-byte records (hot spot of 1e7 particles, 64 x 64 x 32 cells x 200
+// times, an 839 MB tally: 45.0 ms in one window, 50.5 in 20 of the L2's size;
+// word by word it was 105 against 51.6).  Bin averages and detector regions
+// add word by word: the largest window whose [times][cells][4] x 8-byte slice
+// of the tally fits a third of the L2.
 int transient_window_times(const mcbte_transient_params* p) {
   if (p->precision != MCBTE_FP32_TRACE) return p->n_times;
   int wt = p->window_times;
+  if (wt <= 0 && !p->time_average && p->n_regions == 0) return p->n_times;
   if (wt <= 0) {
     int dev = 0, l2 = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess ||

@@ -19,13 +19,12 @@ namespace {
 
 // First measurement index still ahead of the particle: for snapshots the
 // first t_m >= t0, for bin averages the bin [t_{m-1}, t_m) containing t0.
-template <typename R>
-__device__ __forceinline__ void transient_start(Particle<R>& p, const RunCfg& C) {
+__device__ __forceinline__ void transient_start(Particle<double>& p, const RunCfg& C) {
   p.mi = 0;
   if (C.time_average) {
-    while (p.mi < C.n_times && (R)C.t_meas_ps[p.mi] <= p.t) ++p.mi;
+    while (p.mi < C.n_times && C.t_meas_ps[p.mi] <= p.t) ++p.mi;
   } else {
-    while (p.mi < C.n_times && (R)C.t_meas_ps[p.mi] < p.t) ++p.mi;
+    while (p.mi < C.n_times && C.t_meas_ps[p.mi] < p.t) ++p.mi;
   }
 }
 
@@ -167,19 +166,77 @@ __device__ __forceinline__ bool load_state(const uint4* st, uint64_t idx, Partic
   return true;
 }
 
+// Adds val[0..3] to the four words of tally record `rec` (kNoRec: nothing) of
+// every lane.  The four lanes of a quad first transpose their values (two
+// exchanges), so that each reduction instruction adds whole 32-byte records,
+// the quad's lanes side by side: 8 sectors per instruction where a word per
+// lane touched 32, four times each.  Called by all 32 lanes.  A tally has
+// fewer than 2^32 - 1 records on the tracers' grids or `rec` is 64 bits wide.
+constexpr unsigned kNoRec = 0xffffffffu;
+
+template <typename Rec>
+__device__ __forceinline__ void red_records(Rec rec, int val[4], double* snap, int lane) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const bool b0 = (lane & 1) != 0, b1 = (lane & 2) != 0;
+#pragma unroll
+  for (int k = 0; k < 4; k += 2) {
+    const int y = __shfl_xor_sync(kAll, b0 ? val[k] : val[k + 1], 1);
+    if (b0) val[k] = y; else val[k + 1] = y;
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int y = __shfl_xor_sync(kAll, b1 ? val[k] : val[k + 2], 2);
+    if (b1) val[k] = y; else val[k + 2] = y;
+  }
+  long long* q = reinterpret_cast<long long*>(snap) + (lane & 3);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const Rec rr = __shfl_sync(kAll, rec, (lane & ~3) | r);
+    if (rr != (Rec)~(Rec)0) red_s64(q + (size_t)rr * 4, (long long)val[r]);
+  }
+}
+
+// First index in [lo, n] whose measurement time is beyond t_end (closed: t_m <=
+// t_end is not beyond).  Evenly spaced times, the usual request, are hit by
+// the quotient t_end / spacing, checked against its two neighbours; any other
+// case takes a bisection (eight dependent shared-memory reads for 200 times).
+__device__ __forceinline__ int first_beyond(const float* tmeas, int lo, int n, float t_end, bool closed, float inv_dt) {
+  const int g = min(max((int)(t_end * inv_dt), lo), n);
+  auto covered = [&](int m) { return closed ? tmeas[m] <= t_end : tmeas[m] < t_end; };
+  if ((g == n || !covered(g)) && (g == lo || covered(g - 1))) return g;
+  int hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (covered(mid)) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// A warp's flights while their snapshots are shared out (shared memory).
+struct FlightSlots {
+  float4 xt[32];    // position and time at the flight's start
+  float4 uv[32];    // direction, sign x speed
+  int first[32];    // measurement index of the flight's first snapshot - its number in the warp
+};
+
 // Snapshots of a warp's flights, shared out over its 32 lanes.  Lane i
 // takes k_i snapshots this step (measurement indices p.mi .. p.mi + k_i - 1
 // of the flight that starts at p.x at time p.t); a lane's count depends on
 // its flight's length, so a per-lane loop would leave most lanes idle while
 // the longest flights sample.  Here the warp's k_1 + ... + k_32 snapshots are
-// taken 32 at a time: each lane finds the owner of its snapshot by a binary
-// search of the inclusive prefix sums and reads the owner's state by
-// shuffles.  Every lane of the warp must call this (k = 0 for idle lanes).
+// taken 32 at a time.  The flights that have any are written to `fs`, side by
+// side in lane order; where each begins among the 32 of a round is one bit of
+// a mask, so a lane finds its snapshot's flight by a population count.  (A
+// bisection of the prefix sums and ten shuffles of the owner's state took its
+// place before: hot spot of 1e7 particles and 200 snapshots 49.2 ms, now
+// 45.0.)  Every lane of the warp must call this (k = 0 for idle lanes).
 // The arithmetic per snapshot is the per-lane loop's (Eq. sampling, Sec. 3.4).
 __device__ __forceinline__ void warp_snapshots(int k, const Particle<float>& p, const float* tmeas, const float* cinv,
-                                               const RunCfg& C, double* snap) {
+                                               const RunCfg& C, double* snap, FlightSlots& fs) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = (int)(threadIdx.x & 31u);
+  const unsigned some = __ballot_sync(kAll, k > 0);
+  if (!some) return;
   int incl = k;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -187,47 +244,58 @@ __device__ __forceinline__ void warp_snapshots(int k, const Particle<float>& p, 
     if (lane >= o) incl += y;
   }
   const int total = __shfl_sync(kAll, incl, 31);
+  const int excl = incl - k;
+  if (k > 0) {
+    const int r = __popc(some & ((1u << lane) - 1u));
+    fs.xt[r] = make_float4(p.x[0], p.x[1], p.x[2], p.t);
+    fs.uv[r] = make_float4(p.u[0], p.u[1], p.u[2], p.s * p.v);
+    fs.first[r] = p.mi - excl;
+  }
+  __syncwarp();
   const int nx = C.grid[0], ny = C.grid[1], nz = C.grid[2];
   const size_t ncell = (size_t)nx * ny * nz;
+  const bool narrow = ncell * (size_t)C.n_times < (size_t)kNoRec;
+  int before = -1;   // flights that begin before this round, less one
   for (int base = 0; base < total; base += 32) {
+    const int rel = excl - base;
+    const unsigned begins = __reduce_or_sync(kAll, (k > 0 && rel >= 0 && rel < 32) ? 1u << rel : 0u);
     const int j = base + lane;
-    // owner: the first lane whose inclusive sum exceeds j (always in 0..31)
-    int own = 0;
-#pragma unroll
-    for (int st = 16; st >= 1; st >>= 1) {
-      const int v = __shfl_sync(kAll, incl, own + st - 1);
-      if (v <= j) own += st;
-    }
-    const int first = __shfl_sync(kAll, incl - k, own);
-    const int mi0 = __shfl_sync(kAll, p.mi, own);
-    const float x0 = __shfl_sync(kAll, p.x[0], own), x1 = __shfl_sync(kAll, p.x[1], own),
-                x2 = __shfl_sync(kAll, p.x[2], own);
-    const float u0 = __shfl_sync(kAll, p.u[0], own), u1 = __shfl_sync(kAll, p.u[1], own),
-                u2 = __shfl_sync(kAll, p.u[2], own);
-    const float t0 = __shfl_sync(kAll, p.t, own), v = __shfl_sync(kAll, p.v, own),
-                s = __shfl_sync(kAll, p.s, own);
+    unsigned long long rec = ~0ull;
+    int val[4] = {0, 0, 0, 0};
     if (j < total) {
-      const int m = mi0 + (j - first);
-      const float dist = v * (tmeas[m] - t0);
-      const float pm0 = x0 + dist * u0, pm1 = x1 + dist * u1, pm2 = x2 + dist * u2;
+      const int f = before + __popc(begins & (0xffffffffu >> (31 - lane)));
+      const float4 xt = fs.xt[f], uv = fs.uv[f];
+      const int m = fs.first[f] + j;
+      const float sv = uv.w, v = fabsf(sv);
+      const float dist = v * (tmeas[m] - xt.w);
+      const float pm0 = xt.x + dist * uv.x, pm1 = xt.y + dist * uv.y, pm2 = xt.z + dist * uv.z;
       const int ix = min(max((int)floorf(pm0 * cinv[0]), 0), nx - 1);
       const int iy = min(max((int)floorf(pm1 * cinv[1]), 0), ny - 1);
       const int iz = min(max((int)floorf(pm2 * cinv[2]), 0), nz - 1);
-      const size_t c = ((size_t)m * ncell + ((size_t)iz * ny + iy) * nx + ix) * 4;
-      long long* q = reinterpret_cast<long long*>(snap) + c;
-      const float sv = s * v;
-      red_s64(q + 0, s > 0.0f ? 1ll : -1ll);
+      rec = narrow ? (unsigned long long)(((unsigned)m * (unsigned)nz + (unsigned)iz) * (unsigned)ny + (unsigned)iy) * nx + ix
+                   : (unsigned long long)m * ncell + ((size_t)iz * ny + iy) * nx + ix;
       if (v < 1024.0f) {
-        red_s64(q + 1, (long long)__float2int_rn((sv * u0) * kFx));
-        red_s64(q + 2, (long long)__float2int_rn((sv * u1) * kFx));
-        red_s64(q + 3, (long long)__float2int_rn((sv * u2) * kFx));
+        // |s v u_a| <= v (1 + rounding): below 2^30 in fixed point, so the
+        // 32-bit conversion gives the value fx gives
+        val[0] = sv > 0.0f ? 1 : -1;
+        val[1] = __float2int_rn((sv * uv.x) * kFx);
+        val[2] = __float2int_rn((sv * uv.y) * kFx);
+        val[3] = __float2int_rn((sv * uv.z) * kFx);
       } else {
-        red_s64(q + 1, fx(sv * u0));
-        red_s64(q + 2, fx(sv * u1));
-        red_s64(q + 3, fx(sv * u2));
+        // beyond 32 bits in fixed point: this lane adds its own record
+        long long* q = reinterpret_cast<long long*>(snap) + rec * 4;
+        red_s64(q + 0, sv > 0.0f ? 1ll : -1ll);
+        red_s64(q + 1, fx(sv * uv.x));
+        red_s64(q + 2, fx(sv * uv.y));
+        red_s64(q + 3, fx(sv * uv.z));
+        rec = ~0ull;
       }
     }
+    before += __popc(begins);
+    if (narrow) red_records<unsigned>((unsigned)rec, val, snap, lane);
+    else red_records<unsigned long long>(rec, val, snap, lane);
   }
+  __syncwarp();   // the slots are rewritten at the next step
 }
 
 // Time-bin averages of a warp's flights, shared out over its 32 lanes in the
@@ -290,7 +358,8 @@ __device__ __forceinline__ void warp_bin_averages(int k, float t_end, const Part
   }
 }
 
-// Shared memory: the measurement times as float (always), then the relaxation
+// Shared memory: the warps' flight slots (snapshots), the measurement times as
+// float (always), then the relaxation
 // alias records and per-bin constants where the plan has room.
 // TAVG: the run tallies time-bin averages (compiled apart, so that the
 // snapshot variant carries none of that code).
@@ -302,6 +371,12 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
   const int n = M.n;
   const uint4* relax = M.rec_relax;
   const float4* binf = M.binf;
+  // the warps' flight slots first (16-byte aligned), then the measurement times
+  FlightSlots* slots = nullptr;
+  if constexpr (!TAVG) {
+    slots = reinterpret_cast<FlightSlots*>(sp) + (threadIdx.x >> 5);
+    sp += (TPB / 32) * sizeof(FlightSlots);
+  }
   float* tmeas = reinterpret_cast<float*>(sp);
   for (int i = threadIdx.x; i < C.n_times; i += TPB) tmeas[i] = (float)C.t_meas_ps[i];
   sp += ((size_t)C.n_times * sizeof(float) + 15) & ~(size_t)15;
@@ -321,6 +396,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
   float cinv[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) cinv[a] = (float)((double)C.grid[a] / G.L[a]);
+  const float inv_dt = (float)C.n_times / tmeas[C.n_times - 1];
   const uint64_t deadline = *C.t0 + C.budget_ns;
   const unsigned lane = threadIdx.x & 31u;
   const uint2 key = run_key(C);
@@ -352,7 +428,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
             p.pid = (uint32_t)idx;
             p.g = 0;
             emit<float, EXT>(p, G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, true, (float)C.t_max_ps);
-            transient_start(p, C);
+            p.mi = first_beyond(tmeas, 0, C.n_times, p.t, TAVG, inv_dt);   // (bins: the one that holds the emission)
             if (!C.win_last && p.mi >= C.win_end) save_state(A.tstate, idx, p);   // emitted after this window
             else alive = true;
           } else if (load_state(A.tstate, idx, p, M, binf, C)) {
@@ -381,29 +457,17 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           if constexpr (TAVG) {
             // the bins [t_{m-1}, t_m) the flight overlaps: m = p.mi up to the
             // first m whose end t_m lies beyond t_end (the flight's last bin,
-            // where the particle stays), by bisection
-            int lo = p.mi, hi = C.n_times;
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if (tmeas[mid] <= t_end) lo = mid + 1; else hi = mid;
-            }
-            mi_next = lo;
-            k = p.mi < C.n_times ? (lo < C.n_times ? lo : C.n_times - 1) - p.mi + 1 : 0;
+            // where the particle stays)
+            mi_next = first_beyond(tmeas, p.mi, C.n_times, t_end, true, inv_dt);
+            k = p.mi < C.n_times ? (mi_next < C.n_times ? mi_next : C.n_times - 1) - p.mi + 1 : 0;
           } else {
-            // the measurement times in [t, t_end) (closed at t_max): the first
-            // index from p.mi on that is not covered, by bisection
-            int lo = p.mi, hi = C.n_times;
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              const bool cov = fin ? (tmeas[mid] <= t_end) : (tmeas[mid] < t_end);
-              if (cov) lo = mid + 1; else hi = mid;
-            }
-            k = lo - p.mi;
+            // the measurement times in [t, t_end) (closed at t_max)
+            k = first_beyond(tmeas, p.mi, C.n_times, t_end, fin, inv_dt) - p.mi;
           }
         }
       }
       if constexpr (TAVG) warp_bin_averages(k, t_end, p, tmeas, C, A.snap);
-      else warp_snapshots(k, p, tmeas, cinv, C, A.snap);
+      else warp_snapshots(k, p, tmeas, cinv, C, A.snap, *slots);
       bool ended = false;
       if (alive) {
         if (out == STEP_ALIVE) {
@@ -454,7 +518,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
             p.pid = (uint32_t)idx;
             p.g = 0;
             emit<float, EXT>(p, G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, true, (float)C.t_max_ps);
-            transient_start(p, C);
+            p.mi = first_beyond(tmeas, 0, C.n_times, p.t, TAVG, inv_dt);   // (bins: the one that holds the emission)
             if (!C.win_last && p.mi >= C.win_end) save_state(A.tstate, idx, p);   // emitted after this window
             else alive = true;
           } else if (load_state(A.tstate, idx, p, M, binf, C)) {
@@ -489,6 +553,18 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
 
 #endif  // MCBTE_F32
 #if MCBTE_F64
+// q as a double, exactly: for |q| < 2^53 the bits are put together by integer
+// instructions (a conversion takes the FP64 pipe, the finaliser's bottleneck).
+__device__ __forceinline__ double exact_double(long long q) {
+  const unsigned long long m = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
+  if (m == 0ull) return 0.0;
+  if (m >> 53) return (double)q;
+  const int z = __clzll((long long)m);   // 11..63
+  const unsigned long long bits =
+      ((unsigned long long)(1086 - z) << 52) | ((m << (z - 11)) & 0x000fffffffffffffull);
+  return __longlong_as_double((long long)(bits | ((unsigned long long)q & 0x8000000000000000ull)));
+}
+
 // Scale the raw snapshot sums: T = s E_eff / (C V_cell), q = s E_eff V_g / V_cell.
 // `fixed`: the sums are the FP32 path's integers (signed count; flux in
 // 2^-20 nm/ps units), converted here in place.
@@ -498,35 +574,53 @@ __global__ void k_finalize_transient(const GeoRun* geos, MatView M, RunCfg C, Ac
   const double E_eff = G.E_tot / (double)G.n;
   const double Vc = G.V_box / (double)((size_t)C.grid[0] * C.grid[1] * C.grid[2]);
   const size_t total = (size_t)C.n_times * n_cells_total;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    // volume of this entry's detector (its region's split, or the grid cell)
-    double vd = Vc;
-    if (C.n_regs > 0) {
-      const uint32_t det = (uint32_t)(i % n_cells_total);
-      for (int k = 0; k < C.n_regs; ++k)
-        if (det >= C.regs[k].off) vd = C.regs[k].v_det;
+  // (16-byte loads and stores: a caller's tally may be aligned to 8 only)
+  const bool wide = ((reinterpret_cast<uintptr_t>(A.snap) | reinterpret_cast<uintptr_t>(tally)) & 15u) == 0;
+  if (fixed && C.n_regs == 0 && !C.time_average && wide) {
+    // Snapshots on the whole-box grid: one pass over the tally, bound by its
+    // 64 bytes of traffic per entry once the FP64 work is four products and no
+    // quotient (the factors are the same for every entry; the FP64 pipe takes
+    // 1/64 of the FP32 rate).
+    const double kT = E_eff / (M.sums[0] * Vc);
+    const double kq = ((E_eff / Vc) * kFxInv) * 1e3;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+      const longlong2* r = reinterpret_cast<const longlong2*>(A.snap + i * 4);
+      double2* o = reinterpret_cast<double2*>(tally + i * 4);
+      const longlong2 q0 = r[0], q1 = r[1];
+      o[0] = make_double2(kT * exact_double(q0.x), kq * exact_double(q0.y));
+      o[1] = make_double2(kq * exact_double(q1.x), kq * exact_double(q1.y));
     }
-    const double kT = E_eff / (M.sums[0] * vd);
-    const double kq = E_eff / vd;
-    const double* r = A.snap + i * 4;
-    double* o = tally + i * 4;
-    double a0, a1, a2, a3;
-    if (fixed) {
-      const long long* q = reinterpret_cast<const long long*>(r);
-      a0 = C.time_average ? (double)q[0] * kFxInv : (double)q[0];
-      a1 = (double)q[1] * kFxInv;
-      a2 = (double)q[2] * kFxInv;
-      a3 = (double)q[3] * kFxInv;
-    } else {
-      a0 = r[0];
-      a1 = r[1];
-      a2 = r[2];
-      a3 = r[3];
+  } else {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+      // volume of this entry's detector (its region's split, or the grid cell)
+      double vd = Vc;
+      if (C.n_regs > 0) {
+        const uint32_t det = (uint32_t)(i % n_cells_total);
+        for (int k = 0; k < C.n_regs; ++k)
+          if (det >= C.regs[k].off) vd = C.regs[k].v_det;
+      }
+      const double kT = E_eff / (M.sums[0] * vd);
+      const double kq = E_eff / vd;
+      const double* r = A.snap + i * 4;
+      double* o = tally + i * 4;
+      double a0, a1, a2, a3;
+      if (fixed) {
+        const long long* q = reinterpret_cast<const long long*>(r);
+        a0 = C.time_average ? (double)q[0] * kFxInv : (double)q[0];
+        a1 = (double)q[1] * kFxInv;
+        a2 = (double)q[2] * kFxInv;
+        a3 = (double)q[3] * kFxInv;
+      } else {
+        a0 = r[0];
+        a1 = r[1];
+        a2 = r[2];
+        a3 = r[3];
+      }
+      o[0] = kT * a0;
+      o[1] = (kq * a1) * 1e3;
+      o[2] = (kq * a2) * 1e3;
+      o[3] = (kq * a3) * 1e3;
     }
-    o[0] = kT * a0;
-    o[1] = (kq * a1) * 1e3;
-    o[2] = (kq * a2) * 1e3;
-    o[3] = (kq * a3) * 1e3;
   }
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x < 32) {
     // fold the copies of the run counters: a lane per copy, then a warp sum
@@ -588,7 +682,8 @@ namespace {
 template <int TPB, bool EXT, bool TAVG>
 cudaError_t launch_transient_tav(const GeoRun* geos, const MatView& M, const RunCfg& C, const Acc& A, int bps,
                                  cudaStream_t s) {
-  const size_t tm_bytes = ((size_t)C.n_times * sizeof(float) + 15) & ~(size_t)15;
+  const size_t tm_bytes = (((size_t)C.n_times * sizeof(float) + 15) & ~(size_t)15) +
+                          (TAVG ? 0 : (TPB / 32) * sizeof(FlightSlots));
   SmemPlan S = plan_smem_f32(M.n, 1, 0, 0, 200 * 1024 - tm_bytes);
   S.bytes += tm_bytes;
   auto kern = k_transient_f32<TPB, EXT, TAVG>;
