@@ -31,6 +31,10 @@ struct SmemPlan {
   size_t bytes;
 };
 
+// Shared memory a tracer block lays out: 212 of the 227 KB it may have (the
+// rest of the SM's 256 KB is L1, which tables beyond the plan are read through).
+constexpr size_t kTableBytes = 212 * 1024;
+
 SmemPlan plan_smem_f32(int n_bins, int n_geoms, int n_cells, int per_bin, size_t budget, int tail_threads = 0,
                        int grad_acc = 0, int snap_threads = 0);
 

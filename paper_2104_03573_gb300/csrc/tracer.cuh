@@ -973,10 +973,10 @@ struct GradReplay {
 // look).  dry: the counter has run out; with cb >= ce the warp has nothing
 // left to hand out.
 struct WarpRun {
-  uint64_t cb = 0, ce = 0;
-  uint64_t base = 0;   // indices the grid's warps hold from the start
-  unsigned chunk = 32u;
-  bool dry = false;
+  uint64_t cb, ce;
+  uint64_t base;   // indices the grid's warps hold from the start
+  unsigned chunk;
+  bool dry;
 
   // Warps are numbered block by block across the grid (warp 0 of every block
   // first), so a run with fewer chunks than warps spreads over all SMs.
@@ -1012,7 +1012,161 @@ struct WarpRun {
     if (nb + chunk >= total) dry = true;
     return k;
   }
+  // The next consecutive indices, 32 at most: their first one, and how many
+  // (0: the run has no more).  Called by the whole warp.
+  __device__ __forceinline__ uint64_t batch(unsigned lane, unsigned long long* work, uint64_t total, uint64_t deadline,
+                                            int* flags, int* count) {
+    if (cb >= ce && !dry) {
+      unsigned long long nb = 0;
+      if (lane == 0) {
+        nb = base + atomicAdd(work, (unsigned long long)chunk);
+        if (globaltimer_ns() > deadline) atomicOr(flags, 1);
+      }
+      nb = __shfl_sync(0xffffffffu, nb, 0);
+      cb = nb;
+      ce = nb + chunk < total ? nb + chunk : total;
+      if (nb + chunk >= total) dry = true;
+    }
+    const uint64_t first = cb;
+    const uint64_t left = cb < ce ? ce - cb : 0;
+    *count = left < 32 ? (int)left : 32;
+    cb += (unsigned)*count;
+    return first;
+  }
   __device__ __forceinline__ bool empty() const { return dry && cb >= ce; }
+};
+
+// Particles a warp has emitted and not yet handed to a lane, one batch of 32
+// consecutive indices (shared memory, a word per lane and field).  Emission
+// takes three to four Philox blocks and two table reads; emitting for the few
+// lanes that wait left the other lanes idle meanwhile, and waiting for more of
+// them cost lanes too.  A batch is emitted by all 32 lanes at once and a lane
+// refills by a few shared-memory reads.
+template <typename R, bool EXT, bool TR>
+struct EmitBatch {
+  R x[3][32], u[3][32], d_rel[32];
+  R d2[EXT ? 32 : 1];
+  R t[TR ? 32 : 1];
+  uint32_t bin[32];   // bit 31: negative sign
+  uint32_t pid[32];
+  int g[32];
+
+  __device__ __forceinline__ void store(unsigned i, const Particle<R>& p) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      x[a][i] = p.x[a];
+      u[a][i] = p.u[a];
+    }
+    d_rel[i] = p.d_rel;
+    if constexpr (EXT) d2[i] = p.d2;
+    if constexpr (TR) t[i] = p.t;
+    bin[i] = (uint32_t)p.bin | (p.s < R(0) ? 0x80000000u : 0u);
+    pid[i] = p.pid;
+    g[i] = p.g;
+  }
+  __device__ __forceinline__ void load(unsigned i, Particle<R>& p, const MatView& M, const float4* binf) const {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      p.x[a] = x[a][i];
+      p.u[a] = u[a][i];
+    }
+    p.d_rel = d_rel[i];
+    if constexpr (EXT) p.d2 = d2[i];
+    if constexpr (TR) p.t = t[i];
+    const uint32_t b = bin[i];
+    p.bin = (int)(b & 0x7fffffffu);
+    p.s = (b >> 31) ? R(-1) : R(1);
+    p.pid = pid[i];
+    p.g = g[i];
+    particle_reset_counters(p);
+    load_bin(p, M, binf);
+  }
+};
+
+// One particle emitted into slot `lane` of a warp's batch.
+template <typename R, bool EXT, bool TR>
+static __device__ __forceinline__ void emit_slot(EmitBatch<R, EXT, TR>* b, unsigned lane, const GeoRun* geos,
+                                              const uint64_t* offs, int n_geoms, uint64_t idx, const uint4* rec_emit,
+                                              const uint4* rec_init, const float4* binf, int n_bins, int imp,
+                                              uint2 key, R t_max_ps) {
+  MatView M{};
+  M.n = n_bins;
+  M.imp = imp;
+  int lo = 0, hi = n_geoms;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (offs[mid] <= idx) lo = mid; else hi = mid;
+  }
+  const GeoRun& G = geos[lo];
+  Particle<R> p;
+  p.pid = (uint32_t)(idx - offs[lo] + G.pid0);
+  p.g = lo;
+  emit<R, EXT>(p, G, M, rec_emit, rec_init, binf, key.x, key.y, TR, t_max_ps);
+  b->store(lane, p);
+}
+
+// A warp's refill: its run of particle indices, and the batch it emitted last.
+// All of it in shared memory, read once per refill: as registers the
+// warp-uniform state took a dozen of every thread's.  hand_out() gives the
+// lanes in `want` the next particles of the batch and emits new ones as they
+// run out; emit_one(index) emits into the lane's slot, and take(slot, index)
+// is called in each lane that gets one.  Returns whether the run has nothing
+// left for the warp (or its time budget is over).
+template <typename R, bool EXT, bool TR>
+struct Refill {
+  EmitBatch<R, EXT, TR> b;
+  WarpRun run;
+  uint64_t first;   // particle index of the batch's first
+  int next, n;
+
+  // by all lanes of the warp
+  __device__ __forceinline__ void start(unsigned lane, unsigned chunk, uint64_t total, uint64_t deadline, int* flags) {
+    WarpRun r;
+    r.start(chunk, total, deadline, flags);
+    if (lane == 0) {
+      run = r;
+      first = 0;
+      next = n = 0;
+    }
+    __syncwarp();
+  }
+
+  template <class Emit, class Take>
+  __device__ __forceinline__ bool hand_out(unsigned want, unsigned lane, unsigned long long* work, uint64_t total,
+                                           uint64_t deadline, int* flags, Emit emit_one, Take take) {
+    constexpr unsigned kAll = 0xffffffffu;
+    int at = next, cnt_b = n;
+    for (;;) {
+      if (at == cnt_b) {
+        WarpRun r = run;
+        const uint64_t f = r.batch(lane, work, total, deadline, flags, &cnt_b);
+        const int stop = *(volatile int*)flags & 1;
+        if (cnt_b == 0 || __any_sync(kAll, stop)) return true;
+        at = 0;
+        __syncwarp();
+        if (lane == 0) {
+          run = r;
+          first = f;
+          n = cnt_b;
+        }
+        if ((int)lane < cnt_b) emit_one(f + lane);
+        __syncwarp();
+      }
+      const int left = cnt_b - at;
+      const int rank = __popc(want & ((1u << lane) - 1u));
+      const bool mine = ((want >> lane) & 1u) != 0u;
+      if (mine && rank < left) take((unsigned)(at + rank), first + (unsigned)(at + rank));
+      const int cnt = __popc(want);
+      at += cnt < left ? cnt : left;
+      if (cnt <= left) break;
+      want = __ballot_sync(kAll, mine && rank >= left);
+    }
+    __syncwarp();
+    if (lane == 0) next = at;
+    const bool done = at == cnt_b && run.empty();
+    __syncwarp();
+    return done;
+  }
 };
 
 // Philox key of the run: the host seed, or the device-resident one.

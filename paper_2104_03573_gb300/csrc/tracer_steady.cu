@@ -296,7 +296,6 @@ struct ParkRec {
   int bin, n_relax, g;
   uint32_t e, pid;
   long long Xq, Xqper;
-  uint64_t idx;
   // gradient pass
   double Xf, sum_x_res;
   float a, d, pa, pd;
@@ -311,7 +310,7 @@ struct ParkRec {
 };
 
 template <bool GRAD, class GradT>
-__device__ __forceinline__ void park_store(ParkRec* r, const Particle<float>& p, uint64_t idx, const GradT& gr,
+__device__ __forceinline__ void park_store(ParkRec* r, const Particle<float>& p, const GradT& gr,
                                            int n_dirs) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -328,7 +327,6 @@ __device__ __forceinline__ void park_store(ParkRec* r, const Particle<float>& p,
   r->pid = p.pid;
   r->Xq = p.Xq;
   r->Xqper = p.Xqper;
-  r->idx = idx;
   if constexpr (GRAD) {
     r->Xf = gr.Xf;
     r->sum_x_res = gr.sum_x_res;
@@ -357,7 +355,7 @@ __device__ __forceinline__ void park_store(ParkRec* r, const Particle<float>& p,
 }
 
 template <bool GRAD, class GradT>
-__device__ __forceinline__ void park_load(const ParkRec* r, Particle<float>& p, uint64_t& idx, GradT& gr, int n_dirs,
+__device__ __forceinline__ void park_load(const ParkRec* r, Particle<float>& p, GradT& gr, int n_dirs,
                                           const MatView& M, const float4* binf) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -374,7 +372,6 @@ __device__ __forceinline__ void park_load(const ParkRec* r, Particle<float>& p, 
   p.pid = r->pid;
   p.Xq = r->Xq;
   p.Xqper = r->Xqper;
-  idx = r->idx;
   load_bin(p, M, binf);
   if constexpr (GRAD) {
     gr.Xf = r->Xf;
@@ -613,11 +610,15 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
 }
 
 // Every lane owns one particle at a time.  When its particle terminates the
-// lane refills from its warp's run of particle indices (WarpRun: a ballot of
-// the empty lanes, which take consecutive indices of the run; the run is
-// refilled from the global work counter a chunk at a time, one atomic per
-// chunk).  Lanes therefore never idle while work remains, whatever the
-// event-count spread between particles.
+// lane refills from its warp's batch (Refill: 32 particles emitted at once by
+// all lanes into shared memory, from the warp's run of particle indices, which
+// is refilled from the global work counter a chunk at a time).  Lanes therefore
+// never idle while work remains, whatever the event-count spread between
+// particles, and the emission runs with all lanes.  Emitting for the waiting
+// lanes alone took 150 warp instructions a particle; what made room for the
+// batch at 80 registers a thread is that nothing a particle needs once (the
+// lane's book-keeping, the warp's run) stays in registers.  1e7-particle
+// silicon-like slab: 17.98 -> 15.32 ms.
 // TPB is the block size the kernel is compiled for (register budget).
 // GRAD: the gradient pass.  Fused (C.fused): the forward run's tallies,
 // counters and per-particle outputs and the gradient in one pass, each
@@ -663,7 +664,11 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   long long* s_qbin = nullptr;
   long long* s_cP = nullptr;
   long long* s_cD = nullptr;
-  // the tail kernel's per-warp draw slots come first (16-byte aligned), 32 per warp
+  // the warps' emitted batches (main kernel) or the tail kernel's draw slots,
+  // 32 per warp, come first (16-byte aligned)
+  using RefillT = Refill<float, EXT, false>;
+  RefillT& refill = reinterpret_cast<RefillT*>(sp)[threadIdx.x >> 5];
+  if constexpr (!TK) sp += (TPB / 32) * sizeof(RefillT);
   Draw32* slots = nullptr;
   if (TK && S.tail_slots) {
     slots = reinterpret_cast<Draw32*>(sp) + (threadIdx.x & ~31u);
@@ -727,8 +732,17 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
     gr.dirs = C.dirs;
     gr.mvd = C.mvd != 0;
   }
+  // The lane's book-keeping is touched once per particle: kept in local memory
+  // (an address the compiler cannot see through), its 13 registers go to the
+  // event loop.
   ThreadAcct acct;
   acct.reset(-1);
+  auto acct_mem = [&]() -> ThreadAcct* {
+    ThreadAcct* q = &acct;
+    // (no instruction: hides where q points)
+    asm volatile("" : "+l"(q) : : "memory");
+    return q;
+  };
   TallyFxT<CELLS == 2 ? 2 : 4> T;
   T.nc = nc;
   T.ca = C.cell_axis;
@@ -744,7 +758,6 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   };
   bool alive = false;
   bool drained = false;   // no work left for this lane: it idles in the loop until its warp is drained
-  uint64_t idx = 0;
   const GeoRun* G = geos;
   const uint2 key = run_key(C);
   const int refill_min = (C.refill_min > 1 && !TK) ? C.refill_min : 1;
@@ -752,13 +765,15 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   const int tail_max = (TK ? (slots != nullptr && n <= kOneBlockBins) : (MODE == 1 && A.park_cap > 0)) ? C.tail_max : 0;
   const uint64_t n_parked = TK ? min(*(volatile unsigned long long*)A.park_n, (unsigned long long)A.park_cap) : 0;
   bool pool_dry = false;   // the same in every lane: nothing left to hand out
-  WarpRun run;              // main kernel: the warp's particle indices not yet handed out
-  if constexpr (!TK) run.start(C.take_chunk, C.total, deadline, A.flags);
+  if constexpr (!TK) refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
+  // a particle's index in the run
+  auto index_of = [&](const Particle<float>& q) { return offs[q.g] + (q.pid - (uint32_t)geos[q.g].pid0); };
   // the tallies of the lane's geometry
   auto bind = [&](int g) {
-    if (g != acct.g) {
-      acct.flush(A);
-      acct.reset(g);
+    ThreadAcct* am = acct_mem();
+    if (g != am->g) {
+      am->flush(A);
+      am->reset(g);
     }
     G = &geos[g];
     if (CELLS) {
@@ -789,7 +804,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
         if (alive) {
           const unsigned long long slot = base + (unsigned long long)__popc(live & ((1u << lane) - 1u));
           if (slot < A.park_cap) {
-            park_store<GRAD>(reinterpret_cast<ParkRec*>(A.park + slot * A.park_stride), p, idx, gr, C.n_dirs);
+            park_store<GRAD>(reinterpret_cast<ParkRec*>(A.park + slot * A.park_stride), p, gr, C.n_dirs);
             alive = false;
             drained = true;
           }
@@ -846,49 +861,45 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
       const unsigned need = ~(dry | live);
       // refill once enough lanes are idle (or no lane is busy)
       if (need && !pool_dry && (__popc(need) >= refill_min || live == 0u)) {
-        const unsigned cnt = __popc(need);
-        const unsigned rank = __popc(need & ((1u << lane) - 1u));
-        uint64_t k;
-        uint64_t avail;
         if constexpr (TK) {
+          const unsigned cnt = __popc(need);
+          const unsigned rank = __popc(need & ((1u << lane) - 1u));
           const int leader = __ffs(need) - 1;
           unsigned long long base = 0;
           if ((int)lane == leader) base = atomicAdd(A.park_rd, (unsigned long long)cnt);
           base = __shfl_sync(kAll, base, leader);
-          avail = n_parked;
-          if (base + cnt >= avail) pool_dry = true;
-          k = base + rank;
-        } else {
-          k = run.take(need, lane, A.work, C.total, deadline, A.flags);
-          avail = C.total;
-          if (run.empty()) pool_dry = true;
-        }
-        if (!alive && !drained) {
-          if (k >= avail || (*(volatile int*)A.flags & 1)) {
-            drained = true;
-            continue;
-          }
-          if constexpr (TK) {
+          if (base + cnt >= n_parked) pool_dry = true;
+          const uint64_t k = base + rank;
+          if (!alive && !drained) {
+            if (k >= n_parked || (*(volatile int*)A.flags & 1)) {
+              drained = true;
+              continue;
+            }
             // a parked particle, exactly as the main kernel left it
-            park_load<GRAD>(reinterpret_cast<const ParkRec*>(A.park + k * A.park_stride), p, idx, gr, C.n_dirs, M,
+            park_load<GRAD>(reinterpret_cast<const ParkRec*>(A.park + k * A.park_stride), p, gr, C.n_dirs, M,
                             binf);
             bind(p.g);
             if constexpr (GRAD) {
               if (gr.mv.phase) T.qb = nullptr;   // a phantom trace tallies only its own X
             }
-          } else {
-            idx = k;
-            const int g = find_geom(offs, C.n_geoms, idx);
-            bind(g);
-            p.pid = (uint32_t)(idx - offs[g] + G->pid0);
-            p.g = g;
-            emit<float, EXT>(p, *G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, false, 0.0f);
-            if constexpr (GRAD) {
-              gr.init(p.bin);
-              if (!C.fused) gr.Xf = A.X_pp[idx];
-            }
+            alive = true;
           }
-          alive = true;
+        } else {
+          pool_dry = refill.hand_out(
+              need, lane, A.work, C.total, deadline, A.flags,
+              [&](uint64_t k) {
+                emit_slot<float, EXT, false>(&refill.b, lane, geos, offs, C.n_geoms, k, M.rec_emit, M.rec_init, binf, n,
+                                             M.imp, key, 0.0f);
+              },
+              [&](unsigned slot, uint64_t k) {
+                refill.b.load(slot, p, M, binf);
+                bind(p.g);
+                if constexpr (GRAD) {
+                  gr.init(p.bin);
+                  if (!C.fused) gr.Xf = A.X_pp[k];
+                }
+                alive = true;
+              });
         }
       }
       if (!alive) {
@@ -908,20 +919,23 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
     auto account = [&](double X) {
       T.period_end(p);
       const unsigned nev = p.e + 1u;
-      acct.ev += nev;
-      acct.trunc += (out == STEP_TRUNCATED) ? 1u : 0u;
-      acct.maxev = nev > acct.maxev ? nev : acct.maxev;
-      acct.traced += 1u;
-      acct.sxq += p.Xq;
-      acct.sx2 += X * X;
+      // one read and write of the lane's fields, which live in memory (below)
+      ThreadAcct t = const_cast<const ThreadAcct&>(*acct_mem());
+      t.ev += nev;
+      t.trunc += (out == STEP_TRUNCATED) ? 1u : 0u;
+      t.maxev = nev > t.maxev ? nev : t.maxev;
+      t.traced += 1u;
+      t.sxq += p.Xq;
+      t.sx2 += X * X;
       const int sgn = p.s > 0.0f ? 1 : -1;
-      acct.s_emit += sgn;
+      t.s_emit += sgn;
       if (out == STEP_ABSORBED) {
-        acct.s_abs += sgn;
-        acct.absorbed += 1u;
+        t.s_abs += sgn;
+        t.absorbed += 1u;
       }
-      if (A.events_pp) A.events_pp[idx] = nev;
-      if (A.X_pp) A.X_pp[idx] = X;
+      *acct_mem() = t;
+      if (A.events_pp) A.events_pp[index_of(p)] = nev;
+      if (A.X_pp) A.X_pp[index_of(p)] = X;
       if constexpr (EXT) nscat_end(C, p.g, p.n_relax, X);
     };
     if (GRAD) {
@@ -966,8 +980,8 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   }
   const bool one_geom = C.n_geoms == 1;
   if (!GRAD || C.fused) {
-    if (one_geom) s_acct.add(acct);
-    else acct.flush(A);
+    if (one_geom) s_acct.add(*acct_mem());
+    else acct_mem()->flush(A);
   }
   __syncthreads();
   if (threadIdx.x == 0 && one_geom) s_acct.flush(A);
@@ -1172,8 +1186,10 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
                               const Acc& A, int bps, cudaStream_t s) {
   // the gradient kernel keeps no cell tallies, and the per-bin flux only in
   // a fused pass
-  const SmemPlan S = plan_smem_f32(M.n, C.n_geoms, GRAD ? 0 : C.n_cells, (GRAD && !C.fused) ? 0 : C.per_bin,
-                                   200 * 1024, MODE == 2 ? TPB : 0, GRAD ? 1 : 0, (GRAD && C.mvd) ? TPB : 0);
+  constexpr size_t kBatch = MODE == 2 ? 0 : (TPB / 32) * sizeof(Refill<float, EXT, false>);
+  SmemPlan S = plan_smem_f32(M.n, C.n_geoms, GRAD ? 0 : C.n_cells, (GRAD && !C.fused) ? 0 : C.per_bin,
+                                   kTableBytes - kBatch, MODE == 2 ? TPB : 0, GRAD ? 1 : 0, (GRAD && C.mvd) ? TPB : 0);
+  S.bytes += kBatch;
   auto kern = k_steady_f32<CELLS, GRAD, TPB, EXT, MODE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.bytes);
   if (e != cudaSuccess) return e;
