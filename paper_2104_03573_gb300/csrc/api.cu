@@ -483,9 +483,24 @@ int nscat_replicas(int G, int K) {
   return r;
 }
 
+// Copies of the FP64 path's cell and per-bin sums (block b adds to copy b mod
+// copies): every flight adds to a few hundred addresses at most, and FP64
+// reductions on one address take some 25 cycles each (silicon-like slab, 3e5
+// particles, 50 cells: 39.9 ms with one copy, 22.3 with 64 at the same launch
+// shape; gray slab, 1e5: 5.27 and 0.71).  A power of two, up to 64, within
+// 1 MiB, which the finaliser sums in a few tens of microseconds.
+int f64_copies(const mcbte_steady_params* p, int G, int n_bins) {
+  if (p->precision != MCBTE_FP64_PLAIN) return 0;
+  const size_t per = (size_t)G * ((size_t)p->n_cells * 4 + (p->per_bin ? (size_t)n_bins : 0)) * sizeof(double);
+  int r = 64;
+  while (r > 1 && (size_t)r * per > ((size_t)1 << 20)) r >>= 1;
+  return r;
+}
+
+// `f64` copies of the FP64 path's sums, or 0 for the FP32 path's integers.
 SteadyWs layout_steady(char* base, int G, int n, int nc, uint64_t total, bool grad, bool replay, int nd,
                        bool host_out, bool want_ev, bool want_x, bool want_T, bool want_q, bool want_qbin,
-                       uint64_t n_det = 0, int nscat = 0, uint64_t park_cap = 0) {
+                       bool per_bin, int f64, uint64_t n_det = 0, int nscat = 0, uint64_t park_cap = 0) {
   Carve c;
   c.base = base;
   SteadyWs w{};
@@ -493,11 +508,11 @@ SteadyWs layout_steady(char* base, int G, int n, int nc, uint64_t total, bool gr
   w.offs = c.take<uint64_t>(G + 1);
   c.off = (c.off + 255) & ~(size_t)255;
   w.zero_begin = base ? base + c.off : nullptr;
-  w.cellP = nc > 0 ? c.take<double>((size_t)G * nc * 4) : nullptr;
-  w.qbin = c.take<double>((size_t)G * n);
-  w.cellPq = nc > 0 ? c.take<long long>((size_t)G * nc * 4) : nullptr;
-  w.cellDq = nc > 0 ? c.take<long long>((size_t)G * (nc + 1) * 4) : nullptr;
-  w.qbinq = c.take<long long>((size_t)G * n);
+  w.cellP = (nc > 0 && f64) ? c.take<double>((size_t)f64 * G * nc * 4) : nullptr;
+  w.qbin = (per_bin && f64) ? c.take<double>((size_t)f64 * G * n) : nullptr;
+  w.cellPq = (nc > 0 && !f64) ? c.take<long long>((size_t)G * nc * 4) : nullptr;
+  w.cellDq = (nc > 0 && !f64) ? c.take<long long>((size_t)G * (nc + 1) * 4) : nullptr;
+  w.qbinq = (per_bin && !f64) ? c.take<long long>((size_t)G * n) : nullptr;
   w.dsc = c.take<double>((size_t)G * 8);
   w.cnt = c.take<unsigned long long>((size_t)G * 4);
   w.G = grad ? c.take<double>(n) : nullptr;
@@ -630,13 +645,17 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
   // the tail kernel's park buffer when the workspace has room for it (a
   // caller's workspace sized without it still runs, without the tail kernel)
   uint64_t park_cap = park_capacity(p, total);
-  SteadyWs w = layout_steady(nullptr, G, n, nc, total, grad, replay, nd, host_out, out->events_pp, out->X_pp, out->T,
-                             out->q, out->q_bin, det_slots, nscat, park_cap);
+  int f64 = f64_copies(p, G, n);
+  auto layout = [&](char* at) {
+    return layout_steady(at, G, n, nc, total, grad, replay, nd, host_out, out->events_pp, out->X_pp, out->T, out->q,
+                         out->q_bin, p->per_bin != 0, f64, det_slots, nscat, park_cap);
+  };
+  SteadyWs w = layout(nullptr);
   char* base = static_cast<char*>(workspace);
-  if (base && ws_bytes < w.bytes && park_cap) {
+  if (base && ws_bytes < w.bytes && (park_cap || f64 > 1)) {
     park_cap = 0;
-    w = layout_steady(nullptr, G, n, nc, total, grad, replay, nd, host_out, out->events_pp, out->X_pp, out->T, out->q,
-                      out->q_bin, det_slots, nscat, 0);
+    f64 = f64 ? 1 : 0;
+    w = layout(nullptr);
   }
   const size_t need = w.bytes;
   bool own = false;
@@ -647,8 +666,7 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
     return fail(MCBTE_ERR_WORKSPACE, "run_steady: workspace too small");
   }
   char* aligned = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(base) + 255) & ~(uintptr_t)255);
-  w = layout_steady(aligned, G, n, nc, total, grad, replay, nd, host_out, out->events_pp, out->X_pp, out->T, out->q,
-                    out->q_bin, det_slots, nscat, park_cap);
+  w = layout(aligned);
   auto release = [&]() {
     if (own) cudaFreeAsync(base, s);
   };
@@ -687,6 +705,7 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
   C.refill_min = p->refill_threshold;
   C.tail_max = p->tail_lanes == 0 ? 8 : (p->tail_lanes < 0 ? 0 : p->tail_lanes);
   C.fused = fused ? 1 : 0;
+  C.f64_rep = f64;
   C.take_chunk = G > 1 ? 1024u : 256u;   // at most: a warp of a batch stays on one geometry longer
   C.cell_flux_axis = p->cell_flux_axis ? 1 : 0;
   C.ext = (p->n_regions > 0 || nscat > 0) ? 1 : 0;
@@ -820,9 +839,8 @@ mcbte_status mcbte_steady_workspace_size(const mcbte_material* m, const mcbte_ge
   if (!bytes) return fail(MCBTE_ERR_INVALID_ARG, "workspace_size: null bytes");
   SteadyWs w = layout_steady(nullptr, n_geoms, m->n, p->n_cells, total, want_grad != 0,
                              want_grad != 0 && p->precision == MCBTE_FP32_TRACE && !grad_fused(p), n_dirs, false,
-                             false, false, false,
-                             false, false, steady_det_slots(p, m->n), p->nscat_curve ? p->n_scat_max : 0,
-                             park_capacity(p, total));
+                             false, false, false, false, false, p->per_bin != 0, f64_copies(p, n_geoms, m->n),
+                             steady_det_slots(p, m->n), p->nscat_curve ? p->n_scat_max : 0, park_capacity(p, total));
   *bytes = w.bytes;
   return MCBTE_OK;
 }
@@ -1110,10 +1128,10 @@ mcbte_status mcbte_run_steady_noalloc(const mcbte_material* m, const mcbte_geome
   uint64_t total = 0;
   mcbte_status st = check_steady(m, geoms, n_geoms, p, &total);
   if (st != MCBTE_OK) return st;
-  // (the tail kernel's park buffer is used only when it fits as well)
+  // (the tail kernel's park buffer and copies of the FP64 sums are used only when they fit as well)
   const SteadyWs w = layout_steady(nullptr, n_geoms, m->n, p->n_cells, total, false, false, 0, false, false, false,
-                                   false, false, false, steady_det_slots(p, m->n),
-                                   p->nscat_curve ? p->n_scat_max : 0);
+                                   false, false, false, p->per_bin != 0, p->precision == MCBTE_FP64_PLAIN ? 1 : 0,
+                                   steady_det_slots(p, m->n), p->nscat_curve ? p->n_scat_max : 0);
   if (w.bytes > kNoAllocScratchBytes)
     return fail(MCBTE_ERR_WORKSPACE, "run_steady_noalloc: this run needs " + std::to_string(w.bytes) +
                                          " bytes of scratch, above the fixed " +

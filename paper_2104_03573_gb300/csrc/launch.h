@@ -31,6 +31,20 @@ struct SmemPlan {
   size_t bytes;
 };
 
+int sm_count();
+
+// FP64 tracers: one block of six warps per SM, or fewer blocks where the run
+// has no particles for them.  An FP64 warp instruction takes 64 cycles of its
+// scheduler's pipe, one warp nearly fills it, and every further warp makes the
+// longest particle's events wait (silicon-like slab, 3e5 particles, up to 2100
+// events each: 21.9 ms at 16 warps a SM, 17.2 at 8, 16.0 at 6, 15.2 at 4; 2e6
+// particles: 58.9, 54.2, 54.4, 63.0).
+constexpr int kF64Threads = 192;
+inline int f64_blocks(uint64_t total) {
+  const uint64_t most = (uint64_t)sm_count(), need = (total + 31) / 32;   // a warp on every SM first
+  return (int)(need < most ? need : most);
+}
+
 // Shared memory a tracer block lays out: 212 of the 227 KB it may have (the
 // rest of the SM's 256 KB is L1, which tables beyond the plan are read through).
 constexpr size_t kTableBytes = 212 * 1024;
@@ -97,8 +111,6 @@ struct MatBuild {
 };
 
 cudaError_t launch_material_build(const MatBuild& b, cudaStream_t s);
-
-int sm_count();
 
 // Particle indices a warp takes at once: at most `most` (one returning atomic
 // per chunk), and about four chunks per warp of the grid, so that a run of few

@@ -142,14 +142,53 @@ __device__ __forceinline__ double series_log(double x) {
   return (double)ex * 0.6931471805599453 + lm;
 }
 
-// cos(2 pi r), sin(2 pi r), r in [0, 1): octant reduction to theta in
-// [0, pi/4], Taylor polynomials of sin (to theta^15) and cos (to theta^16)
+// m 2^e as a double, exactly, for m < 2^53: the bits are put together by
+// integer instructions.  The FP64 pipe takes 64 cycles a warp instruction on
+// this GPU and bounds every FP64 kernel, while the integer pipes idle, so what
+// is exact in integers is done there.
+__device__ __forceinline__ double exact_scaled(unsigned long long m, int e) {
+  if (m == 0ull) return 0.0;
+  const int z = __clzll((long long)m);   // 11..63
+  return __longlong_as_double(
+      (long long)(((unsigned long long)(1086 - z + e) << 52) | ((m << (z - 11)) & 0x000fffffffffffffull)));
+}
+
+// x with its sign flipped where s < 0 (s is +-1: the product s x, exactly)
+__device__ __forceinline__ double signed_by(double x, double s) {
+  return __longlong_as_double(__double_as_longlong(x) ^ (__double_as_longlong(s) & (long long)0x8000000000000000ull));
+}
+
+// x as a float, truncated, by integer instructions (0 below the float range,
+// infinity above it): for guesses that are checked
+__device__ __forceinline__ float guess_float(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+  const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned mag = e <= 0 ? 0u : (e >= 255 ? 0x7f800000u : ((unsigned)e << 23) | m);
+  return __uint_as_float((hi & 0x80000000u) | mag);
+}
+
+// floor(z / h) clamped to [0, n): a float quotient decides where it lies clear
+// of a whole number, the FP64 quotient elsewhere.
+__device__ __forceinline__ int cell_of(double z, double h, float inv_h, int n) {
+  const float q = guess_float(z) * inv_h;
+  const float f = floorf(q);
+  // the two truncations and the product: below 2^-21 of the quotient
+  const float tol = fabsf(q) * 9.6e-7f + 1e-6f;
+  int c;
+  if (q - f > tol && (f + 1.0f) - q > tol && fabsf(q) < 1e6f) c = (int)f;
+  else c = (int)floor(z / h);
+  return min(max(c, 0), n - 1);
+}
+
+// cos(2 pi r), sin(2 pi r), r = w 2^-32: octant reduction to theta in
+// [0, pi/4] (the octant is the word's top three bits, the rest of it exact in
+// integers), Taylor polynomials of sin (to theta^15) and cos (to theta^16)
 // by Horner from the highest coefficient, then the octant symmetries.
-__device__ __forceinline__ void series_sincos2pi(double r, double* sn, double* cs) {
-  const double t = r * 8.0;
-  const int oct = (int)t;
-  double f = t - (double)oct;
-  if (oct & 1) f = 1.0 - f;
+__device__ __forceinline__ void series_sincos2pi(uint32_t w, double* sn, double* cs) {
+  const int oct = (int)(w >> 29);
+  const uint32_t fr = w & 0x1fffffffu;
+  const double f = exact_scaled((oct & 1) ? 0x20000000u - fr : fr, -29);
   const double th = f * 0.7853981633974483;
   const double t2 = th * th;
   const double sc[8] = {-7.647163731819816e-13, 1.6059043836821613e-10, -2.505210838544172e-08,
@@ -166,32 +205,33 @@ __device__ __forceinline__ void series_sincos2pi(double r, double* sn, double* c
   for (int k = 1; k < 9; ++k) pc = cc[k] + t2 * pc;
   const double S = th * ps;
   const double C = pc;
-  switch (oct & 7) {
-    case 0: *cs = C; *sn = S; break;
-    case 1: *cs = S; *sn = C; break;
-    case 2: *cs = -S; *sn = C; break;
-    case 3: *cs = -C; *sn = S; break;
-    case 4: *cs = -C; *sn = -S; break;
-    case 5: *cs = -S; *sn = -C; break;
-    case 6: *cs = S; *sn = -C; break;
-    default: *cs = C; *sn = -S; break;
-  }
+  // octants: |cos| is C in 0, 3, 4, 7 and S in the others; the signs by bits
+  const bool swap = ((oct + 1) & 2) != 0;
+  const double c = swap ? S : C, t = swap ? C : S;
+  *cs = ((oct + 2) & 4) ? -c : c;
+  *sn = (oct & 4) ? -t : t;
 }
 
 // ------------------------------------------------------------------ real maps
 template <typename R> struct Num;
 
 template <> struct Num<double> {
-  static __device__ __forceinline__ double oc(uint32_t w) { return ((double)w + 1.0) * 2.3283064365386963e-10; }
-  static __device__ __forceinline__ double co(uint32_t w) { return (double)w * 2.3283064365386963e-10; }
-  static __device__ __forceinline__ double mid(uint32_t w) { return ((double)w + 0.5) * 2.3283064365386963e-10; }
+  // (w + 1) 2^-32, w 2^-32, (w + 1/2) 2^-32, and (m + 1) 2^-53 of the 53-bit m
+  static __device__ __forceinline__ double oc(uint32_t w) { return exact_scaled((unsigned long long)w + 1ull, -32); }
+  static __device__ __forceinline__ double co(uint32_t w) { return exact_scaled(w, -32); }
+  static __device__ __forceinline__ double mid(uint32_t w) { return exact_scaled(2ull * w + 1ull, -33); }
+  // 1 - 2 oc(w)
+  static __device__ __forceinline__ double iso_mu(uint32_t w) {
+    const long long k = 0x80000000ll - ((long long)w + 1ll);
+    return signed_by(exact_scaled((unsigned long long)(k < 0 ? -k : k), -31), k < 0 ? -1.0 : 1.0);
+  }
   static __device__ __forceinline__ double oc53(uint32_t lo, uint32_t hi) {
-    const uint64_t m = ((uint64_t)hi << 21) ^ (uint64_t)(lo >> 11);
-    return ((double)m + 1.0) * 1.1102230246251565e-16;
+    const unsigned long long m = (((unsigned long long)hi << 21) ^ (unsigned long long)(lo >> 11)) + 1ull;
+    return (m >> 53) ? 1.0 : exact_scaled(m, -53);
   }
   static __device__ __forceinline__ double log_(double x) { return series_log(x); }
   static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-  static __device__ __forceinline__ void sincos2pi(double r, double* s, double* c) { series_sincos2pi(r, s, c); }
+  static __device__ __forceinline__ void sincos2pi_word(uint32_t w, double* s, double* c) { series_sincos2pi(w, s, c); }
   static __device__ __forceinline__ double fmax_(double a, double b) { return fmax(a, b); }
   static __device__ __forceinline__ double div(double a, double b) { return a / b; }
   static __device__ __forceinline__ double big() { return 1.0e300; }
@@ -211,6 +251,8 @@ template <> struct Num<float> {
   static __device__ __forceinline__ void sincos2pi(float r, float* s, float* c) {
     __sincosf(6.28318530717958647f * r, s, c);
   }
+  static __device__ __forceinline__ void sincos2pi_word(uint32_t w, float* s, float* c) { sincos2pi(co(w), s, c); }
+  static __device__ __forceinline__ float iso_mu(uint32_t w) { return 1.0f - 2.0f * oc(w); }
   static __device__ __forceinline__ float fmax_(float a, float b) { return fmaxf(a, b); }
   // distances for the first hit: the 2-ulp hardware quotient (the particle
   // is set onto the face it hits, so the quotient's last bits move nothing)
@@ -265,7 +307,7 @@ template <typename R>
 __device__ __forceinline__ void dir_about_axis(R u[3], int a, R sgn, R mu, uint32_t wphi) {
   const R s = Num<R>::sqrt_(Num<R>::fmax_(R(0), R(1) - mu * mu));
   R sn, cs;
-  Num<R>::sincos2pi(Num<R>::co(wphi), &sn, &cs);
+  Num<R>::sincos2pi_word(wphi, &sn, &cs);
   put3_cyclic<R>(u, a, sgn * mu, s * cs, s * sn);
 }
 
@@ -288,7 +330,7 @@ template <typename R>
 __device__ __forceinline__ void dir_about_frame(R u[3], const R* f, R mu, uint32_t wphi) {
   const R s = Num<R>::sqrt_(Num<R>::fmax_(R(0), R(1) - mu * mu));
   R sn, cs;
-  Num<R>::sincos2pi(Num<R>::co(wphi), &sn, &cs);
+  Num<R>::sincos2pi_word(wphi, &sn, &cs);
   const R sc = s * cs, ss = s * sn;
   u[0] = (mu * f[0] + sc * f[3]) + ss * f[6];
   u[1] = (mu * f[1] + sc * f[4]) + ss * f[7];
@@ -404,26 +446,66 @@ struct GeoLean {
   __device__ __forceinline__ float L(int a) const { return a == 0 ? Lf[0] : (a == 1 ? Lf[1] : Lf[2]); }
 };
 
+// FP64 box faces.  A float guess of the three face distances, with bounds on
+// its error, finds the face that is nearest beyond doubt, and only that one's
+// FP64 quotient is taken (or none, where every face lies beyond `near`, the
+// distance at which the flight ends in any case); all three where the guess
+// leaves a doubt.  The quotient taken is the one the full scan would take.
+__device__ __forceinline__ void hit_box_f64(const GeoRun& g, const double x[3], const double u[3], double near,
+                                            double* dist, int* face) {
+  float lo[3], hi[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float uf = guess_float(u[a]), Lf = g.Lf[a];
+    const float d = fabsf((uf > 0.0f ? Lf : 0.0f) - guess_float(x[a]));
+    // |L - x| to 4e-7 L (three roundings of at most 2^-23), u to 2^-23
+    const float r = __fdividef(1.0f, fmaxf(fabsf(uf), 1e-30f));
+    lo[a] = fmaxf(d - 4e-7f * Lf, 0.0f) * r * 0.999999f;
+    hi[a] = (d + 4e-7f * Lf) * r * 1.000001f;
+    if (!(fabsf(uf) > 1e-20f)) {   // (also the float zero of a tiny u: left to the full scan)
+      lo[a] = u[a] == 0.0 ? 3e38f : 0.0f;
+      hi[a] = 3e38f;
+    }
+  }
+  const float nf = guess_float(near);
+  const float lmin = fminf(lo[0], fminf(lo[1], lo[2]));
+  if (nf * 1.000001f < lmin) {
+    *dist = 1.0e300;
+    *face = 7;
+    return;
+  }
+  unsigned todo = 7u;
+  if (hi[0] < lo[1] && hi[0] < lo[2]) todo = 1u;
+  else if (hi[1] < lo[0] && hi[1] < lo[2]) todo = 2u;
+  else if (hi[2] < lo[0] && hi[2] < lo[1]) todo = 4u;
+  double best = 1.0e300;
+  int bf = 7;
+  // one quotient in the common case: the axis is a select, not a branch
+  for (unsigned m = todo; m; m &= m - 1u) {
+    const int a = __ffs((int)m) - 1;
+    const double ua = sel3(u, a), xa = sel3(x, a);
+    if (ua == 0.0) continue;
+    const bool up = ua > 0.0;
+    double d = ((up ? g.L[a] : 0.0) - xa) / ua;
+    const int f = up ? axis_max_face(a) : axis_min_face(a);
+    if (d < 0.0) d = 0.0;
+    if (d < best || (d == best && f < bf)) { best = d; bf = f; }
+  }
+  *dist = best;
+  *face = bf;
+}
+
 // First boundary along the ray (faces in the direction of travel, then the
-// pore cylinder); ties go to the lowest paper boundary ID.
+// pore cylinder); ties go to the lowest paper boundary ID.  FP64: a boundary
+// beyond `near` may be reported as none.
 template <typename R, bool EXT = true>
-__device__ __forceinline__ void first_hit(const GeoRun& g, const R x[3], const R u[3], R* dist, int* face) {
+__device__ __forceinline__ void first_hit(const GeoRun& g, const R x[3], const R u[3], R near, R* dist, int* face) {
   R best = Num<R>::big();
   int bf = 7;
   if constexpr (sizeof(R) == 4) {
     hit_box_pore_f32(g, x, u, &best, &bf);
   } else {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      R d;
-      int f;
-      const R La = geo_L<R>(g, a);
-      if (u[a] > R(0)) { d = Num<R>::div(La - x[a], u[a]); f = axis_max_face(a); }
-      else if (u[a] < R(0)) { d = Num<R>::div(R(0) - x[a], u[a]); f = axis_min_face(a); }
-      else continue;
-      if (d < R(0)) d = R(0);
-      if (d < best || (d == best && f < bf)) { best = d; bf = f; }
-    }
+    hit_box_f64(g, x, u, near, &best, &bf);
     if (g.pore) {
       const R cx = (R)g.cx;
       const R cy = (R)g.cy;

@@ -64,6 +64,7 @@ struct RunCfg {
   // nscat_rep copies (a power of two), block b adding to copy b % nscat_rep
   double* nscat_acc;    // [nscat_rep][G][n_scat_max + 1][4]
   int nscat_rep;
+  int f64_rep;          // FP64 path: copies of the cell and per-bin sums (a power of two), block b adding to b % f64_rep
   int det_nb;           // steady detector sums per detector (1) or per detector and bin (n_bins)
   int tail_max;         // FP32 steady tracer: the tail's draw slots serve warps with at most
                         // this many particles in flight once the work counter has run out (0: off)
@@ -167,8 +168,8 @@ constexpr int kSumCopies = 64;
 constexpr int kGradStride = 4 + 2 * kMaxDirs;
 
 struct Acc {
-  double* cellP;              // [G][nc][4]   per-cell sums (FP64 path)
-  double* qbin;               // [G][n_bins]  (FP64 path)
+  double* cellP;              // [f64_rep][G][nc][4] per-cell sums (FP64 path; else null)
+  double* qbin;               // [f64_rep][G][n_bins] (FP64 path; else null)
   long long* cellPq;          // [G][nc][4]   fixed-point partial-cell sums (FP32 path)
   long long* cellDq;          // [G][nc+1][4] difference array of its full-cell sums
   long long* qbinq;           // [G][n_bins]
@@ -247,7 +248,7 @@ __device__ __forceinline__ void resample(Particle<R>& p, const MatView& M, const
                                          uint4 w, uint4 w1, bool lambert, int axis, R sgn,
                                          const R* fr = nullptr) {
   p.bin = alias_draw(rec, M.n, w.x, w.y, w1.x);
-  const R mu = lambert ? Num<R>::sqrt_(Num<R>::oc(w.z)) : R(1) - R(2) * Num<R>::oc(w.z);
+  const R mu = lambert ? Num<R>::sqrt_(Num<R>::oc(w.z)) : Num<R>::iso_mu(w.z);
   if (EXT && axis == 3) dir_about_frame<R>(p.u, fr, mu, w.w);
   else dir_about_axis<R>(p.u, axis, sgn, mu, w.w);
   load_bin(p, M, binf);
@@ -438,8 +439,8 @@ __device__ __forceinline__ void emit_prologue(Particle<R>& p, const GeoRun& g, u
     const R m1 = Num<R>::sqrt_(R(-2) * Num<R>::log_(Num<R>::oc(w3.x)));
     const R m2 = Num<R>::sqrt_(R(-2) * Num<R>::log_(Num<R>::oc(w3.z)));
     R s1, c1, s2, c2;
-    Num<R>::sincos2pi(Num<R>::co(w3.y), &s1, &c1);
-    Num<R>::sincos2pi(Num<R>::co(w3.w), &s2, &c2);
+    Num<R>::sincos2pi_word(w3.y, &s1, &c1);
+    Num<R>::sincos2pi_word(w3.w, &s2, &c2);
     const R nrm[3] = {m1 * c1, m1 * s1, m2 * c2};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -507,6 +508,7 @@ struct TallyPlain {
   double* qb;      // [n_bins], or null
   int nc, ca, ta;
   double h;
+  float inv_h;     // of cell_of
   double* det = nullptr;   // [n_det][4] steady detector-region sums, or null
 
   __device__ __forceinline__ bool has_det() const { return det != nullptr; }
@@ -519,39 +521,48 @@ struct TallyPlain {
 
   __device__ __forceinline__ double X(const Particle<double>& p) const { return p.X; }
 
+  // One quotient per flight, and the cells between the two ends share one
+  // product per component (each crossed cell took a quotient, four comparisons
+  // and eight products of the FP64 pipe).
   __device__ __forceinline__ double segment(Particle<double>& p, double seg) const {
-    const double contrib = (p.s * seg) * sel3(p.u, ta);
+    const double ss = signed_by(seg, p.s);
+    const double contrib = ss * sel3(p.u, ta);
     p.X += contrib;
     if (!cP) return contrib;
     const double z0 = sel3(p.x, ca);
     const double uc = sel3(p.u, ca);
-    const double z1 = z0 + seg * uc;
     if (uc == 0.0) {
-      int c = (int)floor(z0 / h);
-      c = min(max(c, 0), nc - 1);
-      atomicAdd(&cP[c * 4 + 0], (p.s * seg) * p.inv_v);
+      const int c = cell_of(z0, h, inv_h, nc);
+      atomicAdd(&cP[c * 4 + 0], ss * p.inv_v);
 #pragma unroll
-      for (int b = 0; b < 3; ++b) atomicAdd(&cP[c * 4 + 1 + b], (p.s * seg) * p.u[b]);
+      for (int b = 0; b < 3; ++b) atomicAdd(&cP[c * 4 + 1 + b], ss * p.u[b]);
       return contrib;
     }
-    const double zlo = z0 < z1 ? z0 : z1;
-    const double zhi = z0 < z1 ? z1 : z0;
-    const int clo = min(max((int)floor(zlo / h), 0), nc - 1);
-    const int chi = min(max((int)floor(zhi / h), 0), nc - 1);
-    const double au = fabs(uc);
-    for (int c = clo; c <= chi; ++c) {
-      double lo = fmax(zlo, c * h);
-      double hi = fmin(zhi, (c + 1) * h);
-      if (c == nc - 1) hi = zhi;
-      if (c == 0) lo = zlo;
-      const double ov = hi - lo;
-      if (ov <= 0.0) continue;
-      const double l = ov / au;
-      atomicAdd(&cP[c * 4 + 0], (p.s * l) * p.inv_v);
+    const double z1 = z0 + seg * uc;
+    const bool fwd = uc > 0.0;
+    const double zlo = fwd ? z0 : z1;
+    const double zhi = fwd ? z1 : z0;
+    const int clo = cell_of(zlo, h, inv_h, nc);
+    const int chi = cell_of(zhi, h, inv_h, nc);
+    const double k = signed_by(1.0, p.s) / fabs(uc);   // path length per unit of the cell axis, signed
+    const double f[4] = {k * p.inv_v, k * p.u[0], k * p.u[1], k * p.u[2]};
+    add(cP + clo * 4, f, (clo == chi ? zhi : (clo + 1) * h) - zlo);
+    if (clo == chi) return contrib;
+    add(cP + chi * 4, f, zhi - chi * h);
+    if (chi > clo + 1) {
+      const double w[4] = {f[0] * h, f[1] * h, f[2] * h, f[3] * h};
+      for (int c = clo + 1; c < chi; ++c) {
 #pragma unroll
-      for (int b = 0; b < 3; ++b) atomicAdd(&cP[c * 4 + 1 + b], (p.s * l) * p.u[b]);
+        for (int b = 0; b < 4; ++b) atomicAdd(&cP[c * 4 + b], w[b]);
+      }
     }
     return contrib;
+  }
+
+  __device__ __forceinline__ void add(double* a, const double f[4], double ov) const {
+    if (ov <= 0.0) return;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) atomicAdd(&a[b], f[b] * ov);
   }
 
   __device__ __forceinline__ void period_end(Particle<double>& p) const {
@@ -1085,13 +1096,9 @@ struct EmitBatch {
 
 // One particle emitted into slot `lane` of a warp's batch.
 template <typename R, bool EXT, bool TR>
-static __device__ __forceinline__ void emit_slot(EmitBatch<R, EXT, TR>* b, unsigned lane, const GeoRun* geos,
-                                              const uint64_t* offs, int n_geoms, uint64_t idx, const uint4* rec_emit,
-                                              const uint4* rec_init, const float4* binf, int n_bins, int imp,
-                                              uint2 key, R t_max_ps) {
-  MatView M{};
-  M.n = n_bins;
-  M.imp = imp;
+__device__ __forceinline__ void emit_slot(EmitBatch<R, EXT, TR>* b, unsigned lane, const GeoRun* geos,
+                                          const uint64_t* offs, int n_geoms, uint64_t idx, const MatView& M,
+                                          const float4* binf, uint2 key, R t_max_ps) {
   int lo = 0, hi = n_geoms;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -1099,9 +1106,9 @@ static __device__ __forceinline__ void emit_slot(EmitBatch<R, EXT, TR>* b, unsig
   }
   const GeoRun& G = geos[lo];
   Particle<R> p;
-  p.pid = (uint32_t)(idx - offs[lo] + G.pid0);
+  p.pid = (uint32_t)(idx - (n_geoms > 1 ? offs[lo] : 0) + G.pid0);
   p.g = lo;
-  emit<R, EXT>(p, G, M, rec_emit, rec_init, binf, key.x, key.y, TR, t_max_ps);
+  emit<R, EXT>(p, G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, TR, t_max_ps);
   b->store(lane, p);
 }
 
@@ -1242,7 +1249,7 @@ __device__ __forceinline__ int apply_event(Particle<R>& p, const GeoRun& g, cons
         for (int b = 0; b < 3; ++b) p.u[b] = (R)d.iso[b];
       } else {
         const uint4 w = philox(ctr, k0, k1);
-        dir_about_axis<R>(p.u, 2, R(1), R(1) - R(2) * Num<R>::oc(w.z), w.w);
+        dir_about_axis<R>(p.u, 2, R(1), Num<R>::iso_mu(w.z), w.w);
       }
       p.d2 = draw_d2(p, M, binf, k0, k1, src);
       return STEP_ALIVE;
@@ -1350,7 +1357,7 @@ __device__ __forceinline__ int apply_event(Particle<R>& p, const GeoRun& g, cons
       const R mu = Num<R>::sqrt_(Num<R>::oc(w.z));
       const R sn = Num<R>::sqrt_(Num<R>::fmax_(R(0), R(1) - mu * mu));
       R sphi, cphi;
-      Num<R>::sincos2pi(Num<R>::co(w.w), &sphi, &cphi);
+      Num<R>::sincos2pi_word(w.w, &sphi, &cphi);
       const R sc = sn * cphi;
       p.u[0] = mu * nx - sc * ny;
       p.u[1] = mu * ny + sc * nx;
@@ -1425,7 +1432,7 @@ __device__ __forceinline__ int step_steady(Particle<R>& p, const GeoRun& g, cons
   }
   R db;
   int face;
-  first_hit<R, EXT>(g, p.x, p.u, &db, &face);
+  first_hit<R, EXT>(g, p.x, p.u, p.d_rel, &db, &face);
   // nearest of the two scattering clocks and the boundary (Sec. 3.3): the
   // boundary wins ties, the three-phonon clock wins a tie with the two-phonon one
   const bool relax = EXT ? (p.d_rel < db && p.d_rel <= p.d2) : p.d_rel < db;
@@ -1467,6 +1474,19 @@ __device__ __forceinline__ void snap_add(double* snap, size_t c, R s, R sv, cons
   (void)v;
 }
 
+// floor(x / (L / n)) in [0, n), by cell_of's guess where it is clear (six FP64
+// quotients a snapshot elsewhere)
+__device__ __forceinline__ int grid_cell(double x, double L, float Lf, int n) {
+  const float inv_h = __fdividef((float)n, Lf);
+  const float q = guess_float(x) * inv_h;
+  const float f = floorf(q);
+  const float tol = fabsf(q) * 1.5e-6f + 1e-6f;
+  int c;
+  if (q - f > tol && (f + 1.0f) - q > tol && fabsf(q) < 1e5f) c = (int)f;
+  else c = (int)floor(x / (L / (double)n));
+  return min(max(c, 0), n - 1);
+}
+
 // `tmeas`: the measurement times in ps (FP64 path: the global array; FP32
 // path: a float copy in shared memory).  `cinv`: cells per nm along x, y, z
 // (FP32 path only; the FP64 path divides by the cell size, the CPU reference form).
@@ -1478,10 +1498,10 @@ __device__ __forceinline__ int step_transient(Particle<R>& p, const GeoRun& g, c
   if (p.e + 1u >= C.max_events) return STEP_TRUNCATED;
   R db;
   int face;
-  first_hit<R, EXT>(g, p.x, p.u, &db, &face);
   const R v = p.v;
   const R tmax = (R)C.t_max_ps;
   const R d_end = (tmax - p.t) * v;
+  first_hit<R, EXT>(g, p.x, p.u, d_end < p.d_rel ? d_end : p.d_rel, &db, &face);
   bool fin = false, relax = false, relax2 = false;
   R seg;
   if (d_end <= p.d_rel && d_end <= db && (!EXT || d_end <= p.d2)) { fin = true; seg = d_end; }
@@ -1540,9 +1560,9 @@ __device__ __forceinline__ int step_transient(Particle<R>& p, const GeoRun& g, c
     for (int a = 0; a < 3; ++a) pm[a] = p.x[a] + dist * p.u[a];
     int ix, iy, iz;
     if constexpr (sizeof(R) == 8) {
-      ix = (int)floor(pm[0] / (geo_L<R>(g, 0) / (R)nx));
-      iy = (int)floor(pm[1] / (geo_L<R>(g, 1) / (R)ny));
-      iz = (int)floor(pm[2] / (geo_L<R>(g, 2) / (R)nz));
+      ix = grid_cell(pm[0], g.L[0], g.Lf[0], nx);
+      iy = grid_cell(pm[1], g.L[1], g.Lf[1], ny);
+      iz = grid_cell(pm[2], g.L[2], g.Lf[2], nz);
     } else {
       ix = (int)floorf(pm[0] * cinv[0]);
       iy = (int)floorf(pm[1] * cinv[1]);

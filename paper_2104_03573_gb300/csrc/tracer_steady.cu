@@ -76,107 +76,22 @@ struct GradPick { using type = On; };
 template <class On>
 struct GradPick<false, On> { using type = GradOff; };
 
-#if MCBTE_F64
-// ------------------------------------------------------------------ FP64 plain
-template <bool CELLS, bool GRAD>
-__global__ void __launch_bounds__(256) k_steady_fp64(const GeoRun* __restrict__ geos, const uint64_t* __restrict__ offs,
-                                                     MatView M, RunCfg C, Acc A) {
-  const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= C.total) return;
-  const int g = find_geom(offs, C.n_geoms, idx);
-  const GeoRun& G = geos[g];
-  const uint64_t deadline = *C.t0 + C.budget_ns;
-  Particle<double> p;
-  p.pid = (uint32_t)(idx - offs[g] + G.pid0);
-  p.g = g;
-  const uint2 key = run_key(C);
-  if (globaltimer_ns() > deadline) {   // over budget before this particle started
-    atomicOr(A.flags, 1);
-    return;
-  }
-  emit<double>(p, G, M, M.rec_emit, M.rec_init, nullptr, key.x, key.y, false, 0.0);
-  typename GradPick<GRAD, GradList>::type gr;
-  if constexpr (GRAD) gr.mvd = C.mvd != 0;
-  if (GRAD) gr.init(p.bin);
-  TallyPlain T;
-  T.cP = CELLS ? A.cellP + (size_t)g * C.n_cells * 4 : nullptr;
-  T.qb = C.per_bin ? A.qbin + (size_t)g * M.n : nullptr;
-  T.nc = C.n_cells;
-  T.ca = C.cell_axis;
-  T.ta = C.tally_axis;
-  T.h = CELLS ? G.L[C.cell_axis] / (double)C.n_cells : 1.0;
-  T.det = C.n_regs > 0 ? A.det_raw : nullptr;
-  int out;
-  for (;;) {
-    out = step_steady<double, typename GradPick<GRAD, GradList>::type, TallyPlain>(p, G, M, M.rec_relax, nullptr, C,
-                                                                                 key.x, key.y, T, gr);
-    if (out != STEP_ALIVE) break;
-    if ((p.e & 1023u) == 0u && globaltimer_ns() > deadline) {
-      atomicOr(A.flags, 1);
-      out = STEP_TRUNCATED;
-      break;
-    }
-  }
-  T.period_end(p);
-  const unsigned long long nev = (unsigned long long)p.e + 1ull;
-  atomicAdd(&A.cnt[g * 4 + 0], nev);
-  if (out == STEP_TRUNCATED) atomicAdd(&A.cnt[g * 4 + 1], 1ull);
-  atomicMax(&A.cnt[g * 4 + 2], nev);
-  atomicAdd(&A.cnt[g * 4 + 3], 1ull);
-  atomicAdd(&A.dsc[g * 8 + 0], p.X);
-  atomicAdd(&A.dsc[g * 8 + 1], p.X * p.X);
-  atomicAdd(&A.dsc[g * 8 + 2], p.s);
-  if (out == STEP_ABSORBED) {
-    atomicAdd(&A.dsc[g * 8 + 3], p.s);
-    atomicAdd(&A.dsc[g * 8 + 7], 1.0);
-  }
-  if (A.events_pp) A.events_pp[idx] = (uint32_t)nev;
-  if (A.X_pp) A.X_pp[idx] = p.X;
-  nscat_end(C, g, p.n_relax, p.X);
-  if constexpr (GRAD) {
-    grad_finish(gr, p.X, g, C, A, M);
-    if (C.mvd && gr.mv.sel > 0u) {
-      // measure-valued d/dp_pore: the particle again from its emission, the
-      // chosen pore hit's branch flipped; nothing is tallied but its X
-      const double Xn = p.X;
-      gr.mv.start_phantom();
-      emit<double>(p, G, M, M.rec_emit, M.rec_init, nullptr, key.x, key.y, false, 0.0);
-      TallyPlain Tq;
-      Tq.cP = nullptr;
-      Tq.qb = nullptr;
-      Tq.nc = C.n_cells;
-      Tq.ca = C.cell_axis;
-      Tq.ta = C.tally_axis;
-      Tq.h = 1.0;
-      Tq.det = nullptr;
-      for (;;) {
-        const int o = step_steady<double, GradList, TallyPlain>(p, G, M, M.rec_relax, nullptr, C, key.x, key.y, Tq, gr);
-        if (o != STEP_ALIVE) break;
-        if ((p.e & 1023u) == 0u && globaltimer_ns() > deadline) {
-          atomicOr(A.flags, 1);
-          break;
-        }
-      }
-      const double D = gr.mv.score(Xn, p.X);
-      double* gs = grad_copy(A);
-      atomicAdd(gs + 1, D);
-      atomicAdd(gs + 2, D * D);
-    }
-  }
-}
-#endif  // MCBTE_F64
-
-#if MCBTE_F32
-// ------------------------------------------------------------------ FP32 persistent
 // Per-thread book-keeping of finished particles (integer / fixed-point
 // fields, few registers), flushed to the geometry's global accumulators when
 // the thread moves to another geometry and at exit.
+// SX: the tally's type, 2^-20 nm whole numbers (FP32 path, exact) or FP64 nm.
+__device__ __forceinline__ double tally_nm(long long x) { return (double)x * kFxInv; }
+__device__ __forceinline__ double tally_nm(double x) { return x; }
+__device__ __forceinline__ void tally_add(long long* a, long long x) { red_s64(a, x); }
+__device__ __forceinline__ void tally_add(double* a, double x) { atomicAdd(a, x); }
+
+template <typename SX>
 struct ThreadAcct {
   int g;
   unsigned traced, trunc, absorbed, maxev;
   int s_emit, s_abs;
   unsigned long long ev;
-  long long sxq;      // sum of X in units of 2^-20 nm (exact)
+  SX sx;              // sum of X
   double sx2;
 
   __device__ __forceinline__ void reset(int gg) {
@@ -184,8 +99,22 @@ struct ThreadAcct {
     traced = trunc = absorbed = maxev = 0u;
     s_emit = s_abs = 0;
     ev = 0ull;
-    sxq = 0;
+    sx = SX(0);
     sx2 = 0.0;
+  }
+  // a particle with tally X (x in the tally's type) ended with `out` after nev events
+  __device__ __forceinline__ void end(int out, unsigned nev, int sgn, SX x, double X) {
+    ev += nev;
+    trunc += (out == STEP_TRUNCATED) ? 1u : 0u;
+    maxev = nev > maxev ? nev : maxev;
+    traced += 1u;
+    sx += x;
+    sx2 += X * X;
+    s_emit += sgn;
+    if (out == STEP_ABSORBED) {
+      s_abs += sgn;
+      absorbed += 1u;
+    }
   }
   __device__ __forceinline__ void flush(const Acc& A) const {
     if (g < 0 || traced == 0u) return;
@@ -193,7 +122,7 @@ struct ThreadAcct {
     if (trunc) atomicAdd(&A.cnt[g * 4 + 1], (unsigned long long)trunc);
     atomicMax(&A.cnt[g * 4 + 2], (unsigned long long)maxev);
     atomicAdd(&A.cnt[g * 4 + 3], (unsigned long long)traced);
-    atomicAdd(&A.dsc[g * 8 + 0], (double)sxq * kFxInv);
+    atomicAdd(&A.dsc[g * 8 + 0], tally_nm(sx));
     atomicAdd(&A.dsc[g * 8 + 1], sx2);
     atomicAdd(&A.dsc[g * 8 + 2], (double)s_emit);
     if (absorbed) {
@@ -208,20 +137,24 @@ struct ThreadAcct {
 // addresses (about 0.4 ms, whatever the run's length: a gray slab of 1e5
 // particles 502 us, 35 us without them); a warp's lanes are summed by
 // shuffles, the block's warps here, and a block adds once.
+template <typename SX>
 struct BlockAcct {
   unsigned long long ev, trunc, maxev, traced;
-  long long sxq, s_emit, s_abs, absorbed;
+  long long s_emit, s_abs, absorbed;
+  SX sx;
   double sx2;
 
   __device__ __forceinline__ void reset() {
     ev = trunc = maxev = traced = 0ull;
-    sxq = s_emit = s_abs = absorbed = 0;
+    s_emit = s_abs = absorbed = 0;
+    sx = SX(0);
     sx2 = 0.0;
   }
   // called by all 32 lanes of a warp
-  __device__ __forceinline__ void add(const ThreadAcct& t) {
+  __device__ __forceinline__ void add(const ThreadAcct<SX>& t) {
     constexpr unsigned kAll = 0xffffffffu;
-    unsigned long long ev_w = t.ev, sx_w = (unsigned long long)t.sxq;
+    unsigned long long ev_w = t.ev;
+    SX sx_w = t.sx;
     long long se = t.s_emit, sa = t.s_abs;
     double s2 = t.sx2;
     unsigned long long tr = t.traced;
@@ -241,7 +174,7 @@ struct BlockAcct {
     if (tc) atomicAdd(&trunc, (unsigned long long)tc);
     atomicMax(&maxev, (unsigned long long)mx);
     atomicAdd(&traced, tr);
-    red_s64(&sxq, (long long)sx_w);
+    tally_add(&sx, sx_w);
     atomicAdd(&sx2, s2);
     red_s64(&s_emit, se);
     if (ab) {
@@ -256,7 +189,7 @@ struct BlockAcct {
     if (trunc) atomicAdd(&A.cnt[1], trunc);
     atomicMax(&A.cnt[2], maxev);
     atomicAdd(&A.cnt[3], traced);
-    atomicAdd(&A.dsc[0], (double)sxq * kFxInv);
+    atomicAdd(&A.dsc[0], tally_nm(sx));
     atomicAdd(&A.dsc[1], sx2);
     atomicAdd(&A.dsc[2], (double)s_emit);
     if (absorbed) {
@@ -266,6 +199,123 @@ struct BlockAcct {
   }
 };
 
+#if MCBTE_F64
+// ------------------------------------------------------------------ FP64 plain
+// Persistent: a warp emits 32 particles at a time and a lane that is done
+// takes the next one (Refill).  The FP64 pipe bounds the kernel, a warp
+// instruction taking 64 cycles whether one lane or 32 are active; with a
+// thread per particle 3.8 lanes were, most of them waiting for their warp's
+// longest particle (silicon-like slab, 3e5 particles: 80.1 ms, now 16.0).
+template <bool CELLS, bool GRAD>
+__global__ void __launch_bounds__(kF64Threads, 1) k_steady_fp64(const GeoRun* __restrict__ geos,
+                                                                const uint64_t* __restrict__ offs, MatView M, RunCfg C,
+                                                                Acc A) {
+  __shared__ Refill<double, true, false> s_refill[kF64Threads / 32];
+  __shared__ BlockAcct<double> s_acct;
+  if (threadIdx.x == 0) s_acct.reset();
+  __syncthreads();
+  constexpr unsigned kAll = 0xffffffffu;
+  const unsigned lane = threadIdx.x & 31u;
+  const uint64_t deadline = *C.t0 + C.budget_ns;
+  const uint2 key = run_key(C);
+  Refill<double, true, false>& refill = s_refill[threadIdx.x >> 5];
+  refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
+  Particle<double> p;
+  using GradT = typename GradPick<GRAD, GradList>::type;
+  GradT gr;
+  if constexpr (GRAD) gr.mvd = C.mvd != 0;
+  ThreadAcct<double> acct;
+  acct.reset(-1);
+  TallyPlain T;
+  T.nc = C.n_cells;
+  T.ca = C.cell_axis;
+  T.ta = C.tally_axis;
+  T.cP = T.qb = nullptr;
+  T.h = 1.0;
+  T.inv_h = 1.0f;
+  T.det = nullptr;
+  const size_t copy = blockIdx.x & (unsigned)(C.f64_rep - 1);   // of the cell and per-bin sums
+  const GeoRun* G = geos;
+  double X_nom = 0.0;   // gradient: the nominal trace's tally while the phantom runs
+  bool alive = false, pool_dry = false;
+  for (;;) {
+    const unsigned need = __ballot_sync(kAll, !alive);
+    if (need && !pool_dry) {
+      pool_dry = refill.hand_out(
+          need, lane, A.work, C.total, deadline, A.flags,
+          [&](uint64_t k) {
+            emit_slot<double, true, false>(&refill.b, lane, geos, offs, C.n_geoms, k, M, nullptr, key, 0.0);
+          },
+          [&](unsigned slot, uint64_t) {
+            refill.b.load(slot, p, M, nullptr);
+            if (p.g != acct.g) {
+              acct.flush(A);
+              acct.reset(p.g);
+            }
+            G = &geos[p.g];
+            if (CELLS) {
+              T.cP = A.cellP + (copy * C.n_geoms + p.g) * C.n_cells * 4;
+              T.h = G->L[C.cell_axis] / (double)C.n_cells;
+              T.inv_h = (float)C.n_cells / G->Lf[C.cell_axis];
+            }
+            T.qb = C.per_bin ? A.qbin + (copy * C.n_geoms + p.g) * M.n : nullptr;
+            T.det = C.n_regs > 0 ? A.det_raw : nullptr;
+            if (GRAD) gr.init(p.bin);
+            alive = true;
+          });
+    }
+    if (!__any_sync(kAll, alive)) {
+      if (pool_dry) break;
+      continue;
+    }
+    if (!alive) continue;
+    int out = step_steady<double, GradT, TallyPlain>(p, *G, M, M.rec_relax, nullptr, C, key.x, key.y, T, gr);
+    if (out == STEP_ALIVE && (p.e & 1023u) == 0u && globaltimer_ns() > deadline) {
+      atomicOr(A.flags, 1);
+      out = STEP_TRUNCATED;
+    }
+    if (out == STEP_ALIVE) continue;
+    if constexpr (GRAD) {
+      if (gr.mv.phase) {   // the phantom trace: nothing is tallied but its X
+        const double D = gr.mv.score(X_nom, p.X);
+        double* gs = grad_copy(A);
+        atomicAdd(gs + 1, D);
+        atomicAdd(gs + 2, D * D);
+        alive = false;
+        continue;
+      }
+    }
+    T.period_end(p);
+    acct.end(out, p.e + 1u, p.s > 0.0 ? 1 : -1, p.X, p.X);
+    if (A.events_pp || A.X_pp) {
+      const uint64_t idx = offs[p.g] + (p.pid - (uint32_t)G->pid0);
+      if (A.events_pp) A.events_pp[idx] = p.e + 1u;
+      if (A.X_pp) A.X_pp[idx] = p.X;
+    }
+    nscat_end(C, p.g, p.n_relax, p.X);
+    alive = false;
+    if constexpr (GRAD) {
+      grad_finish(gr, p.X, p.g, C, A, M);
+      if (C.mvd && gr.mv.sel > 0u) {
+        // measure-valued d/dp_pore: the particle again from its emission, the
+        // chosen pore hit's branch flipped
+        X_nom = p.X;
+        gr.mv.start_phantom();
+        T.cP = T.qb = T.det = nullptr;
+        emit<double>(p, *G, M, M.rec_emit, M.rec_init, nullptr, key.x, key.y, false, 0.0);
+        alive = true;
+      }
+    }
+  }
+  if (C.n_geoms == 1) s_acct.add(acct);
+  else acct.flush(A);
+  __syncthreads();
+  if (threadIdx.x == 0 && C.n_geoms == 1) s_acct.flush(A);
+}
+#endif  // MCBTE_F64
+
+#if MCBTE_F32
+// ------------------------------------------------------------------ FP32 persistent
 // Gradient pass: the open period closes at the particle's end (X = X_f; a
 // fused pass adds its listed periods' a X_f too), then the resampling and
 // specularity terms and the directional values.
@@ -426,7 +476,7 @@ __device__ __forceinline__ int trace_slots(Particle<float>& p, const GeoRun& g, 
     if (p.e + 1u >= C.max_events) return STEP_TRUNCATED;
     float db;
     int face;
-    if constexpr (EXT) first_hit<float, EXT>(g, p.x, p.u, &db, &face);
+    if constexpr (EXT) first_hit<float, EXT>(g, p.x, p.u, p.d_rel, &db, &face);
     else hit_box_pore_f32(gl, p.x, p.u, &db, &face);
     const bool relax = EXT ? (p.d_rel < db && p.d_rel <= p.d2) : p.d_rel < db;
     const bool relax2 = EXT && !relax && p.d2 < db;
@@ -708,7 +758,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
     s_cD = s_cP + (size_t)nc * 4;
     for (int i = threadIdx.x; i < nc * 4 + (nc + 1) * 4; i += blockDim.x) s_cP[i] = 0;
   }
-  __shared__ BlockAcct s_acct;
+  __shared__ BlockAcct<long long> s_acct;
   if (threadIdx.x == 0) s_acct.reset();
   __syncthreads();
 
@@ -735,10 +785,10 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   // The lane's book-keeping is touched once per particle: kept in local memory
   // (an address the compiler cannot see through), its 13 registers go to the
   // event loop.
-  ThreadAcct acct;
+  ThreadAcct<long long> acct;
   acct.reset(-1);
-  auto acct_mem = [&]() -> ThreadAcct* {
-    ThreadAcct* q = &acct;
+  auto acct_mem = [&]() -> ThreadAcct<long long>* {
+    ThreadAcct<long long>* q = &acct;
     // (no instruction: hides where q points)
     asm volatile("" : "+l"(q) : : "memory");
     return q;
@@ -770,7 +820,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   auto index_of = [&](const Particle<float>& q) { return offs[q.g] + (q.pid - (uint32_t)geos[q.g].pid0); };
   // the tallies of the lane's geometry
   auto bind = [&](int g) {
-    ThreadAcct* am = acct_mem();
+    ThreadAcct<long long>* am = acct_mem();
     if (g != am->g) {
       am->flush(A);
       am->reset(g);
@@ -888,8 +938,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
           pool_dry = refill.hand_out(
               need, lane, A.work, C.total, deadline, A.flags,
               [&](uint64_t k) {
-                emit_slot<float, EXT, false>(&refill.b, lane, geos, offs, C.n_geoms, k, M.rec_emit, M.rec_init, binf, n,
-                                             M.imp, key, 0.0f);
+                emit_slot<float, EXT, false>(&refill.b, lane, geos, offs, C.n_geoms, k, M, binf, key, 0.0f);
               },
               [&](unsigned slot, uint64_t k) {
                 refill.b.load(slot, p, M, binf);
@@ -920,19 +969,8 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
       T.period_end(p);
       const unsigned nev = p.e + 1u;
       // one read and write of the lane's fields, which live in memory (below)
-      ThreadAcct t = const_cast<const ThreadAcct&>(*acct_mem());
-      t.ev += nev;
-      t.trunc += (out == STEP_TRUNCATED) ? 1u : 0u;
-      t.maxev = nev > t.maxev ? nev : t.maxev;
-      t.traced += 1u;
-      t.sxq += p.Xq;
-      t.sx2 += X * X;
-      const int sgn = p.s > 0.0f ? 1 : -1;
-      t.s_emit += sgn;
-      if (out == STEP_ABSORBED) {
-        t.s_abs += sgn;
-        t.absorbed += 1u;
-      }
+      ThreadAcct<long long> t = *acct_mem();
+      t.end(out, nev, p.s > 0.0f ? 1 : -1, p.Xq, X);
       *acct_mem() = t;
       if (A.events_pp) A.events_pp[index_of(p)] = nev;
       if (A.X_pp) A.X_pp[index_of(p)] = X;
@@ -1026,24 +1064,31 @@ __global__ void k_finalize_steady(const GeoRun* geos, MatView M, RunCfg C, Acc A
     const int b = (int)warp;
     const double Vc = G.V_box / (double)nc;
     const double k = b == 0 ? E_eff / (C_tot * Vc) : E_eff / Vc;
-    const double* P = A.cellP + (size_t)g * nc * 4;
-    const long long* Pq = A.cellPq + (size_t)g * nc * 4;
-    const long long* Dq = A.cellDq + (size_t)g * (nc + 1) * 4;
+    const size_t stride = (size_t)C.n_geoms * nc * 4;   // between copies (FP64 path)
     long long carry = 0;
     for (int c0 = 0; c0 < nc; c0 += 32) {
       const int c = c0 + (int)lane;
       const bool in = c < nc;
-      long long run = in ? Dq[c * 4 + b] : 0;
-      const long long pq = in ? Pq[c * 4 + b] : 0;
-      const double pd = in ? P[c * 4 + b] : 0.0;
+      double v = 0.0;
+      if (C.f64_rep) {
+        if (in) {
+          const double* P = A.cellP + ((size_t)g * nc + c) * 4 + b;
+#pragma unroll 8
+          for (int r = 0; r < C.f64_rep; ++r) v += P[r * stride];
+        }
+      } else {
+        const size_t at = ((size_t)g * nc + c) * 4 + b;
+        long long run = in ? A.cellDq[at + (size_t)g * 4] : 0;   // [G][nc + 1][4]
+        const long long pq = in ? A.cellPq[at] : 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, run, o);
-        if ((int)lane >= o) run += y;
+        for (int o = 1; o < 32; o <<= 1) {
+          const long long y = __shfl_up_sync(0xffffffffu, run, o);
+          if ((int)lane >= o) run += y;
+        }
+        run += carry;
+        carry = __shfl_sync(0xffffffffu, run, 31);
+        v = (double)(pq + run) * kFxInv;
       }
-      run += carry;
-      carry = __shfl_sync(0xffffffffu, run, 31);
-      const double v = pd + (double)(pq + run) * kFxInv;
       if (!in) continue;
       if (b == 0 && O.T) O.T[(size_t)g * nc + c] = (k * v) * 1e-12;
       if (b > 0 && O.q) O.q[((size_t)g * nc + c) * 3 + (b - 1)] = (k * v) * 1e-9;
@@ -1102,7 +1147,15 @@ __global__ void k_finalize_steady(const GeoRun* geos, MatView M, RunCfg C, Acc A
     const double kb = E_eff / G.V_solid;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const size_t j = (size_t)g * n + i;
-      O.q_bin[j] = (kb * (A.qbin[j] + (double)A.qbinq[j] * kFxInv)) * 1e-9;
+      double v = 0.0;
+      if (C.f64_rep) {
+        const size_t stride = (size_t)C.n_geoms * n;
+#pragma unroll 8
+        for (int r = 0; r < C.f64_rep; ++r) v += A.qbin[r * stride + j];
+      } else {
+        v = (double)A.qbinq[j] * kFxInv;
+      }
+      O.q_bin[j] = (kb * v) * 1e-9;
     }
   }
   if (threadIdx.x == 128) {   // (a warp the cells leave free)
@@ -1173,8 +1226,11 @@ __global__ void k_dirs_dot_pi(const double* dirs, int nd, MatView M, double* dpi
 template <bool CELLS, bool GRAD>
 cudaError_t launch_f64(const GeoRun* geos, const uint64_t* offs, const MatView& M, const RunCfg& C, const Acc& A,
                        cudaStream_t s) {
-  const uint64_t blocks = (C.total + 255) / 256;
-  k_steady_fp64<CELLS, GRAD><<<(unsigned)blocks, 256, 0, s>>>(geos, offs, M, C, A);
+  auto kern = k_steady_fp64<CELLS, GRAD>;
+  const int blocks = f64_blocks(C.total);
+  RunCfg R = C;
+  R.take_chunk = take_chunk(C.total, (uint64_t)blocks * (kF64Threads / 32), 256u);
+  kern<<<blocks, kF64Threads, 0, s>>>(geos, offs, M, R, A);
   return cudaGetLastError();
 }
 #endif  // MCBTE_F64

@@ -20,29 +20,13 @@ namespace {
 // First measurement index still ahead of the particle: for snapshots the
 // first t_m >= t0, for bin averages the bin [t_{m-1}, t_m) containing t0.
 __device__ __forceinline__ void transient_start(Particle<double>& p, const RunCfg& C) {
-  p.mi = 0;
-  if (C.time_average) {
-    while (p.mi < C.n_times && C.t_meas_ps[p.mi] <= p.t) ++p.mi;
-  } else {
-    while (p.mi < C.n_times && C.t_meas_ps[p.mi] < p.t) ++p.mi;
+  int lo = 0, hi = C.n_times;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    const double tm = C.t_meas_ps[mid];
+    if (C.time_average ? tm <= p.t : tm < p.t) lo = mid + 1; else hi = mid;
   }
-}
-
-template <typename R>
-__device__ __forceinline__ void transient_finish(const Particle<R>& p, int out, uint64_t idx, const Acc& A) {
-  const unsigned long long nev = (unsigned long long)p.e + 1ull;
-  unsigned long long* cnt = A.cnt + sum_copy() * 4;
-  double* dsc = A.dsc + sum_copy() * 8;
-  atomicAdd(cnt + 0, nev);
-  if (out == STEP_TRUNCATED) atomicAdd(cnt + 1, 1ull);
-  atomicMax(cnt + 2, nev);
-  atomicAdd(cnt + 3, 1ull);
-  atomicAdd(dsc + 2, (double)p.s);
-  if (out == STEP_ABSORBED) {
-    atomicAdd(dsc + 3, (double)p.s);
-    atomicAdd(dsc + 7, 1.0);
-  }
-  if (A.events_pp) A.events_pp[idx] = (uint32_t)nev;
+  p.mi = lo;
 }
 
 // The run counters of a warp's finished particles, spread over its lanes:
@@ -88,32 +72,55 @@ struct WarpAcct {
 };
 
 #if MCBTE_F64
-__global__ void __launch_bounds__(256) k_transient_fp64(const GeoRun* __restrict__ geos, MatView M, RunCfg C, Acc A) {
-  const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= C.total) return;
+// Persistent, like k_steady_fp64: 32 particles emitted at a time, a lane that
+// is done refills.
+__global__ void __launch_bounds__(kF64Threads, 1) k_transient_fp64(const GeoRun* __restrict__ geos, MatView M, RunCfg C,
+                                                                   Acc A) {
+  __shared__ Refill<double, true, true> s_refill[kF64Threads / 32];
+  constexpr unsigned kAll = 0xffffffffu;
+  const unsigned lane = threadIdx.x & 31u;
   const GeoRun& G = geos[0];
   const uint64_t deadline = *C.t0 + C.budget_ns;
-  Particle<double> p;
-  p.pid = (uint32_t)idx;
-  p.g = 0;
   const uint2 key = run_key(C);
-  if (globaltimer_ns() > deadline) {   // over budget before this particle started
-    atomicOr(A.flags, 1);
-    return;
-  }
-  emit<double>(p, G, M, M.rec_emit, M.rec_init, nullptr, key.x, key.y, true, C.t_max_ps);
-  transient_start(p, C);
-  int out;
+  Refill<double, true, true>& refill = s_refill[threadIdx.x >> 5];
+  refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
+  Particle<double> p;
+  p.e = 0u;
+  p.s = 0.0;
+  WarpAcct acct;
+  bool alive = false, pool_dry = false;
   for (;;) {
-    out = step_transient<double>(p, G, M, M.rec_relax, nullptr, C, key.x, key.y, A.snap, C.t_meas_ps, nullptr);
-    if (out != STEP_ALIVE) break;
-    if ((p.e & 1023u) == 0u && globaltimer_ns() > deadline) {
-      atomicOr(A.flags, 1);
-      out = STEP_TRUNCATED;
-      break;
+    const unsigned need = __ballot_sync(kAll, !alive);
+    if (need && !pool_dry) {
+      pool_dry = refill.hand_out(
+          need, lane, A.work, C.total, deadline, A.flags,
+          [&](uint64_t k) {
+            emit_slot<double, true, true>(&refill.b, lane, geos, nullptr, 1, k, M, nullptr, key, C.t_max_ps);
+          },
+          [&](unsigned slot, uint64_t) {
+            refill.b.load(slot, p, M, nullptr);
+            transient_start(p, C);
+            alive = true;
+          });
     }
+    if (!__any_sync(kAll, alive)) {
+      if (pool_dry) break;
+      continue;
+    }
+    int out = STEP_ALIVE;
+    if (alive) {
+      out = step_transient<double>(p, G, M, M.rec_relax, nullptr, C, key.x, key.y, A.snap, C.t_meas_ps, nullptr);
+      if (out == STEP_ALIVE && (p.e & 1023u) == 0u && globaltimer_ns() > deadline) {
+        atomicOr(A.flags, 1);
+        out = STEP_TRUNCATED;
+      }
+    }
+    const bool ended = alive && out != STEP_ALIVE;
+    if (ended && A.events_pp) A.events_pp[p.pid] = p.e + 1u;
+    acct.add(ended, out, p.e, (float)p.s, lane);
+    if (ended) alive = false;
   }
-  transient_finish(p, out, idx, A);
+  acct.flush(lane, A);
 }
 
 #endif  // MCBTE_F64
@@ -446,7 +453,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           out = STEP_TRUNCATED;
         } else {
           float db;
-          first_hit<float, EXT>(G, p.x, p.u, &db, &face);
+          first_hit<float, EXT>(G, p.x, p.u, p.d_rel, &db, &face);
           const float tmax = (float)C.t_max_ps;
           const float d_end = (tmax - p.t) * p.v;
           if (d_end <= p.d_rel && d_end <= db && (!EXT || d_end <= p.d2)) { fin = true; seg = d_end; }
@@ -669,8 +676,10 @@ __global__ void k_finalize_transient(const GeoRun* geos, MatView M, RunCfg C, Ac
 cudaError_t launch_transient(int precision, const GeoRun* geos, const MatView& M, const RunCfg& C, const Acc& A,
                              int threads, int bps, cudaStream_t s) {
   if (precision == MCBTE_FP64_PLAIN) {
-    const uint64_t blocks = (C.total + 255) / 256;
-    k_transient_fp64<<<(unsigned)blocks, 256, 0, s>>>(geos, M, C, A);
+    const int blocks = f64_blocks(C.total);
+    RunCfg R = C;
+    R.take_chunk = take_chunk(C.total, (uint64_t)blocks * (kF64Threads / 32), 256u);
+    k_transient_fp64<<<blocks, kF64Threads, 0, s>>>(geos, M, R, A);
     return cudaGetLastError();
   }
   return launch_transient_f32(geos, M, C, A, threads > 0 ? threads : 1024, bps, s);
