@@ -22,15 +22,21 @@ LIB = os.path.join(HERE, "libmcbte.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 # (source, extra flags, fused multiply-add allowed)
+# FP32 tracers: denormals flushed.  Every quantity they hold (nm, ps, direction
+# cosines, factors) is 0 or far above 1e-38, so the results are the same bits,
+# and the hardware approximations (reciprocal, square roots, logarithm, sines)
+# come without the instructions that handle denormals (41-44 -> 18 cycles each
+# on a lone particle's chain).
+FTZ = "--ftz=true"
 UNITS = [
     ("tables.cu", [], False),
     ("setup.cu", [], False),
     ("api.cu", [], False),
     ("tracer_steady.cu", ["-DMCBTE_F64=1"], False),
-    ("tracer_steady.cu", ["-DMCBTE_F32=1", "-DMCBTE_F32_PART=0"], True),
-    ("tracer_steady.cu", ["-DMCBTE_F32=1", "-DMCBTE_F32_PART=1"], True),
+    ("tracer_steady.cu", ["-DMCBTE_F32=1", "-DMCBTE_F32_PART=0", FTZ], True),
+    ("tracer_steady.cu", ["-DMCBTE_F32=1", "-DMCBTE_F32_PART=1", FTZ], True),
     ("tracer_transient.cu", ["-DMCBTE_F64=1"], False),
-    ("tracer_transient.cu", ["-DMCBTE_F32=1"], True),
+    ("tracer_transient.cu", ["-DMCBTE_F32=1", FTZ], True),
 ]
 
 

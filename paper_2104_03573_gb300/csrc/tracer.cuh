@@ -866,6 +866,9 @@ struct GradReplay {
   // whole, and the per-flight scalars above would go with it.
   double* dv;           // [kMaxDirs] per direction: sum over closed periods of value x dirs[bin]
   bool mvd;             // measure-valued d/dp (set by the kernel)
+  // scores of a specular and a diffuse pore hit, 1/p and -1/(1-p) (set by the
+  // kernel: two FP64 quotients, which every pore hit waited for)
+  float sc_spec, sc_diff;
   bool fused;           // one pass (set by the kernel)
   int np;               // fused: listed periods
   int* lb;              // [kFusedPeriods] fused: their bins
@@ -964,9 +967,9 @@ struct GradReplay {
     sum_x_res += Xnow;
   }
   template <class Word>
-  __device__ __forceinline__ bool pore_branch(bool spec, double p, double, Word word) {
+  __device__ __forceinline__ bool pore_branch(bool spec, double, double, Word word) {
     if (mvd) return mv.branch(spec, word);
-    pa += spec ? (float)(1.0 / p) : (float)(-1.0 / (1.0 - p));
+    pa += spec ? sc_spec : sc_diff;
     return spec;
   }
   __device__ __forceinline__ double resample_term(double X) const { return (double)n_res * X - sum_x_res; }

@@ -11,6 +11,7 @@
 #include <atomic>
 
 #include "launch.h"
+#include "tail.cuh"
 
 #ifndef MCBTE_F64
 #define MCBTE_F64 0
@@ -452,79 +453,20 @@ __device__ __forceinline__ void park_load(const ParkRec* r, Particle<float>& p, 
   }
 }
 
-// The tail kernel's events of one live particle from its precomputed draws:
-// slot0 holds the draws of event p.e + 1, and the slots end with event
-// e_last.  A flight that ends on a periodic face draws nothing, so it is
-// handled here without the event dispatch (the same operations as
-// apply_event's periodic branch: ++e, the clocks run down, the particle moves
-// to the opposite face).  Without the extended physics the box and the pore
-// are read once into registers (GeoLean: the per-event geometry then costs no
-// load on the particle's dependent chain) and a flight that ends on a box
-// face takes apply_event's FP32 face branch here, from the register copy;
-// relaxations, pore hits and, with the extended physics, every non-periodic
-// event go through apply_event with their slot.  Returns at the particle's
-// end, or ALIVE once the slots are used up.
-template <class Grad, class Tally, bool EXT>
+// The tail kernel's events of one live particle from its precomputed draws
+// where trace_lean does not go (extended physics with detector regions, the
+// N_scat_max curve, or walls in a batch of geometries): slot0 holds the draws
+// of event p.e + 1, and the slots end with event e_last.  Returns at the
+// particle's end, or ALIVE once the slots are used up.
+template <class Grad, class Tally>
 __device__ __forceinline__ int trace_slots(Particle<float>& p, const GeoRun& g, const MatView& M, const uint4* relax_tab,
                                            const float4* binf, const RunCfg& C, uint32_t k0, uint32_t k1,
-                                           const Tally& T, Grad& gr, const Draw32* slot0, uint32_t e_last,
-                                           uint64_t deadline, int* flags) {
+                                           const Tally& T, Grad& gr, const DrawLean* slot0, uint32_t e_last) {
   const uint32_t e0 = p.e;
-  GeoLean gl;
-  if constexpr (!EXT) gl.load(g);
   for (;;) {
-    if (p.e + 1u >= C.max_events) return STEP_TRUNCATED;
-    float db;
-    int face;
-    if constexpr (EXT) first_hit<float, EXT>(g, p.x, p.u, p.d_rel, &db, &face);
-    else hit_box_pore_f32(gl, p.x, p.u, &db, &face);
-    const bool relax = EXT ? (p.d_rel < db && p.d_rel <= p.d2) : p.d_rel < db;
-    const bool relax2 = EXT && !relax && p.d2 < db;
-    const float seg = relax ? p.d_rel : (relax2 ? p.d2 : db);
-    double Xb = 0.0;
-    if (Grad::on) Xb = T.X(p);
-    const auto c = T.segment(p, seg);
-    if constexpr (EXT) {
-      if (C.n_regs > 0 && T.has_det()) region_steady<float>(p, seg, C, T);
-    }
-    if (Grad::on) gr.flight(relax, (double)Num<float>::div(seg, p.lam), Xb, c);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) p.x[a] = p.x[a] + seg * p.u[a];
-    const bool box = !relax && !relax2 && face < 6;
-    const int ty = box ? (EXT ? g.type[face] : gl.type(face)) : -1;
-    int out = STEP_ALIVE;
-    if (ty == MCBTE_FACE_PERIODIC) {
-      ++p.e;
-      p.d_rel = p.d_rel - seg;
-      if constexpr (EXT) p.d2 = p.d2 - seg;
-      const int a = face_axis(face);
-      put3<float>(p.x, a, face_is_max(face) ? 0.0f : (EXT ? geo_L<float>(g, a) : gl.L(a)));
-    } else if (!EXT && box) {
-      // apply_event's FP32 face branch (isothermal: absorbed; adiabatic:
-      // specular or Lambertian by the slot's draws, then a select)
-      ++p.e;
-      p.d_rel = p.d_rel - seg;
-      const int a = face_axis(face);
-      const int mx = face_is_max(face);
-      put3<float>(p.x, a, mx ? gl.L(a) : 0.0f);
-      if (ty == MCBTE_FACE_ISOTHERMAL) return STEP_ABSORBED;
-      const Draw32& d = slot0[p.e - 1u - e0];
-      const bool spec_f = (uint64_t)d.wx < g.pthr[face];
-      float ud[3];
-      put3_cyclic<float>(ud, a, mx ? -d.lam[0] : d.lam[0], d.lam[1], d.lam[2]);
-      const float flip = -sel3(p.u, a);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) p.u[b] = spec_f ? (b == a ? flip : p.u[b]) : ud[b];
-    } else {
-      out = apply_event<float, Grad, Tally, EXT, DrawSlot>(p, g, M, relax_tab, binf, C, k0, k1, relax, relax2, face,
-                                                           seg, T, gr, Grad::on ? T.X(p) : 0.0,
-                                                           DrawSlot{slot0 + (p.e - e0)});
-      if (out != STEP_ALIVE) return out;
-    }
-    if ((p.e & 255u) == 0u && globaltimer_ns() > deadline) {
-      atomicOr(flags, 1);
-      return STEP_TRUNCATED;
-    }
+    const int out = step_steady<float, Grad, Tally, true, DrawSlot>(p, g, M, relax_tab, binf, C, k0, k1, T, gr,
+                                                                    DrawSlot{slot0 + (p.e - e0)});
+    if (out != STEP_ALIVE) return out;
     if (p.e >= e_last) return STEP_ALIVE;
   }
 }
@@ -537,8 +479,8 @@ __device__ __forceinline__ int trace_slots(Particle<float>& p, const GeoRun& g, 
 template <class Tally>
 __device__ __forceinline__ int trace_unfolded(Particle<float>& p, const GeoRun& g, const MatView& M,
                                               const uint4* relax_tab, const float4* binf, const RunCfg& C, uint32_t k0,
-                                              uint32_t k1, const Tally& T, const Draw32* slot0, uint32_t e_last,
-                                              uint64_t deadline, int* flags, unsigned um) {
+                                              uint32_t k1, const Tally& T, const DrawLean* slot0, uint32_t e_last,
+                                              unsigned um) {
   const uint32_t e0 = p.e;
   const uint32_t nslots = e_last - e0;
   GeoLean gl;
@@ -585,76 +527,6 @@ __device__ __forceinline__ int trace_unfolded(Particle<float>& p, const GeoRun& 
                                                                             DrawSlotOr{slot});
       if (out != STEP_ALIVE) return out;
     }
-    if ((p.e & 255u) == 0u && globaltimer_ns() > deadline) {
-      atomicOr(flags, 1);
-      return STEP_TRUNCATED;
-    }
-    if (p.e >= e_last) return STEP_ALIVE;
-  }
-}
-
-// trace_unfolded for a box whose only faces left are the pair across axis W
-// (the other two axes unfolded: a film): the flight's first hit is that
-// pair's, and the pair's types and specular thresholds sit in registers.
-// The same operations as hit_box_pore_f32 with those axes skipped and as
-// apply_event's face branch, hence the same bits as step_steady.
-template <int W, class Tally>
-__device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, const MatView& M,
-                                          const uint4* relax_tab, const float4* binf, const RunCfg& C, uint32_t k0,
-                                          uint32_t k1, const Tally& T, const Draw32* slot0, uint32_t e_last,
-                                          uint64_t deadline, int* flags, unsigned um) {
-  const uint32_t e0 = p.e;
-  const uint32_t nslots = e_last - e0;
-  float Lf[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) Lf[a] = g.Lf[a];
-  const int f_lo = axis_min_face(W), f_hi = axis_max_face(W);
-  const bool iso_lo = g.type[f_lo] == MCBTE_FACE_ISOTHERMAL, iso_hi = g.type[f_hi] == MCBTE_FACE_ISOTHERMAL;
-  const uint64_t th_lo = g.pthr[f_lo], th_hi = g.pthr[f_hi];
-  GradOff off;
-  for (;;) {
-    if (p.e + 1u >= C.max_events) return STEP_TRUNCATED;
-    const float uw = p.u[W];
-    const bool up = uw > 0.0f;
-    const bool ok = uw != 0.0f;
-    const float d0 = Num<float>::div((up ? Lf[W] : 0.0f) - p.x[W], uw);
-    const float db = ok ? (d0 < 0.0f ? 0.0f : d0) : Num<float>::big();
-    const bool relax = p.d_rel < db;
-    const float seg = relax ? p.d_rel : db;
-    T.segment(p, seg);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) p.x[a] = p.x[a] + seg * p.u[a];
-    const uint32_t n = fold_periodic(p.x, Lf, um);
-    if (n >= C.max_events - 1u - p.e) {
-      p.e = C.max_events - 1u;
-      return STEP_TRUNCATED;
-    }
-    p.e += n;
-    const uint32_t si = p.e - e0;
-    const Draw32* slot = si < nslots ? slot0 + si : nullptr;
-    if (!relax && ok) {
-      // a wall of the pair
-      ++p.e;
-      p.d_rel = p.d_rel - seg;
-      p.x[W] = up ? Lf[W] : 0.0f;
-      if (up ? iso_hi : iso_lo) return STEP_ABSORBED;
-      const Draw32 d = DrawSlotOr{slot}.sub0(make_uint4(p.pid, (uint32_t)p.g, p.e, 0u), k0, k1, relax_tab, M.n);
-      const bool spec_f = (uint64_t)d.wx < (up ? th_hi : th_lo);
-      float ud[3];
-      put3_cyclic<float>(ud, W, up ? -d.lam[0] : d.lam[0], d.lam[1], d.lam[2]);
-      const float flip = -p.u[W];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) p.u[b] = spec_f ? (b == W ? flip : p.u[b]) : ud[b];
-    } else {
-      const int out = apply_event<float, GradOff, Tally, false, DrawSlotOr>(p, g, M, relax_tab, binf, C, k0, k1,
-                                                                            relax, false, ok ? (up ? f_hi : f_lo) : 7,
-                                                                            seg, T, off, 0.0, DrawSlotOr{slot});
-      if (out != STEP_ALIVE) return out;
-    }
-    if ((p.e & 255u) == 0u && globaltimer_ns() > deadline) {
-      atomicOr(flags, 1);
-      return STEP_TRUNCATED;
-    }
     if (p.e >= e_last) return STEP_ALIVE;
   }
 }
@@ -691,10 +563,10 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
 // rest of the run.  The tail kernel (MODE 2, launched next on the same
 // stream) takes the parked particles instead of emitting new ones; once none
 // is left, a warp with at most C.tail_max particles in flight computes the
-// draws of their next events on all 32 lanes at once (one Draw32 per lane,
-// the warp's 32 slots shared out over its live particles, 32 / 2^ceil(log2
+// draws of their next events on all 32 lanes at once (two DrawLean per lane,
+// the warp's 64 slots shared out over its live particles, 64 / 2^ceil(log2
 // live) events each) and every live lane traces that many events reading its
-// slots (DrawSlot), so its dependent chain per event holds the geometry and
+// slots (tail.cuh), so its dependent chain per event holds the geometry and
 // the tallies only.  The draws are the inline path's, the parked state is
 // resumed as it was: trajectories and tallies are bit for bit those of a
 // single kernel.
@@ -719,10 +591,10 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   using RefillT = Refill<float, EXT, false>;
   RefillT& refill = reinterpret_cast<RefillT*>(sp)[threadIdx.x >> 5];
   if constexpr (!TK) sp += (TPB / 32) * sizeof(RefillT);
-  Draw32* slots = nullptr;
+  DrawLean* slots = nullptr;
   if (TK && S.tail_slots) {
-    slots = reinterpret_cast<Draw32*>(sp) + (threadIdx.x & ~31u);
-    sp += (size_t)TPB * sizeof(Draw32);
+    slots = reinterpret_cast<DrawLean*>(sp) + (size_t)(threadIdx.x >> 5) * kTailSlots;
+    sp += (size_t)(TPB / 32) * kTailSlots * sizeof(DrawLean);
   }
   // then the pore-hit snapshots (16-byte aligned), four int4 per thread
   int4* snaps = nullptr;
@@ -760,6 +632,10 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   }
   __shared__ BlockAcct<long long> s_acct;
   if (threadIdx.x == 0) s_acct.reset();
+  // the tail's walls (one geometry)
+  __shared__ WallLean s_walls[TK && EXT ? kMaxInner : 1];
+  if (TK && EXT && C.n_geoms == 1)
+    for (int i = threadIdx.x; i < kMaxInner; i += blockDim.x) s_walls[i].set(geos[0], i);
   __syncthreads();
 
   const unsigned lane = threadIdx.x & 31u;
@@ -781,6 +657,8 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
     gr.n_bins = n;
     gr.dirs = C.dirs;
     gr.mvd = C.mvd != 0;
+    gr.sc_spec = (float)(1.0 / geos[0].p_pore);
+    gr.sc_diff = (float)(-1.0 / (1.0 - geos[0].p_pore));
   }
   // The lane's book-keeping is touched once per particle: kept in local memory
   // (an address the compiler cannot see through), its 13 registers go to the
@@ -861,49 +739,67 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
         }
         continue;   // lanes the buffer could not take trace on with the next votes (park_cap reached)
       } else {
-        // log2 of the slots per particle: 5 - ceil(log2(nlive)), so nlive << sh <= 32
-        const int sh = 5 - (32 - __clz(nlive - 1));
-        const int r = (int)(lane >> sh);                                        // the live particle this lane draws for
-        unsigned mm = live;
-        for (int i = 0; i < r && mm; ++i) mm &= mm - 1u;
-        const int owner = mm ? __ffs(mm) - 1 : 0;
-        const uint32_t e_o = __shfl_sync(kAll, p.e, owner);
-        const uint32_t pid_o = __shfl_sync(kAll, p.pid, owner);
-        const int g_o = __shfl_sync(kAll, p.g, owner);
-        if (r < nlive) {
-          Draw32 d;
-          uint4 ctr = make_uint4(pid_o, (uint32_t)g_o, e_o + 1u + (lane & ((1u << sh) - 1u)), 0u);
-          draw_words(d, philox(ctr, key.x, key.y), relax, n);
-          d.E2 = 0.0f;
-          d.mv_lo = d.mv_hi = 0u;
-          if (EXT && M.imp) {
-            ctr.w = 256u;
-            d.E2 = draw_e2(philox(ctr, key.x, key.y));
+        // log2 of the slots per particle: nlive << sh <= kTailSlots
+        const int sh = (kTailSlots == 64 ? 6 : 5) - (32 - __clz(nlive - 1));
+        for (unsigned i = lane; i < (unsigned)kTailSlots; i += 32u) {
+          const int r = (int)(i >> sh);   // the live particle slot i belongs to
+          unsigned mm = live;
+          for (int k = 0; k < r && mm; ++k) mm &= mm - 1u;
+          const int owner = mm ? __ffs(mm) - 1 : 0;
+          const uint32_t e_o = __shfl_sync(kAll, p.e, owner);
+          const uint32_t pid_o = __shfl_sync(kAll, p.pid, owner);
+          const int g_o = __shfl_sync(kAll, p.g, owner);
+          float s_o = 0.0f;
+          if constexpr (UNF) s_o = __shfl_sync(kAll, p.s, owner);
+          if (r < nlive) {
+            DrawLean d;
+            uint4 ctr = make_uint4(pid_o, (uint32_t)g_o, e_o + 1u + (i & ((1u << sh) - 1u)), 0u);
+            draw_words(d, philox(ctr, key.x, key.y), relax, n);
+            d.E2 = 0.0f;
+            d.mv_lo = d.mv_hi = 0u;
+            if (EXT && M.imp) {
+              ctr.w = 256u;
+              d.E2 = draw_e2(philox(ctr, key.x, key.y));
+            }
+            if (GRAD && C.mvd) {
+              ctr.w = 257u;
+              const uint4 w7 = philox(ctr, key.x, key.y);
+              d.mv_lo = w7.x;
+              d.mv_hi = w7.y;
+            }
+            draw_lean(d, geos[g_o], binf, EXT);
+            if constexpr (UNF) {
+              const unsigned um_o = unfold_mask<GradT>(geos[g_o], C);
+              const int W = um_o == 3u ? 2 : (um_o == 5u ? 1 : (um_o == 6u ? 0 : -1));
+              if (W >= 0) film_flight(d, geos[g_o], W, s_o, T.ta);
+            }
+            slots[i] = d;
           }
-          if (GRAD && C.mvd) {
-            ctr.w = 257u;
-            const uint4 w7 = philox(ctr, key.x, key.y);
-            d.mv_lo = w7.x;
-            d.mv_hi = w7.y;
-          }
-          slots[lane] = d;
         }
         __syncwarp();
         if (alive) {
-          const Draw32* s0 = slots + (__popc(live & ((1u << lane) - 1u)) << sh);
+          const DrawLean* s0 = slots + (__popc(live & ((1u << lane) - 1u)) << sh);
           const unsigned um = UNF ? unfold_mask<GradT>(*G, C) : 0u;
-          const uint32_t e_l = p.e + (1u << sh);
+          const uint32_t e_f = p.e, e_l = p.e + (1u << sh);
           if (UNF && um == 3u)
-            out = trace_film<2>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, deadline, A.flags, um);
+            out = trace_film<2>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l);
           else if (UNF && um == 5u)
-            out = trace_film<1>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, deadline, A.flags, um);
+            out = trace_film<1>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l);
           else if (UNF && um == 6u)
-            out = trace_film<0>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, deadline, A.flags, um);
+            out = trace_film<0>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l);
           else if (UNF && um)
-            out = trace_unfolded(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, deadline, A.flags, um);
+            out = trace_unfolded(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, um);
+          else if (EXT && (C.n_regs > 0 || C.nscat_acc || (C.n_geoms > 1 && G->n_inner > 0)))
+            out = trace_slots<GradT, decltype(T)>(p, *G, M, relax, binf, C, key.x, key.y, T, gr, s0, e_l);
+          else if (G->pore)
+            out = trace_lean<GradT, decltype(T), EXT, (CELLS > 0), true>(p, *G, s_walls, M, binf, C, T, gr, s0, e_l);
           else
-            out = trace_slots<GradT, decltype(T), EXT>(p, *G, M, relax, binf, C, key.x, key.y, T, gr, s0,
-                                                        p.e + (1u << sh), deadline, A.flags);
+            out = trace_lean<GradT, decltype(T), EXT, (CELLS > 0), false>(p, *G, s_walls, M, binf, C, T, gr, s0, e_l);
+          // (the time budget every 256 events)
+          if (out == STEP_ALIVE && ((e_f ^ p.e) >> 8) != 0u && globaltimer_ns() > deadline) {
+            atomicOr(A.flags, 1);
+            out = STEP_TRUNCATED;
+          }
         }
         __syncwarp();   // the slots are rewritten in the next round
       }
@@ -1317,7 +1213,7 @@ SmemPlan plan_smem_f32(int n_bins, int n_geoms, int n_cells, int per_bin, size_t
   // constants (every relaxation), the cell tallies (every flight), the
   // per-bin flux (every relaxation period), the gradient accumulator (every
   // period of a gradient pass); each is placed while room remains, then the
-  // tail's draw slots (one Draw32 per thread), then the pore-hit snapshots
+  // tail's draw slots (kTailSlots DrawLean per warp), then the pore-hit snapshots
   // of the measure-valued d/dp (64 bytes per thread).
   SmemPlan S{0, 0, 0, 0, 0, 0, 0, 0};
   size_t used = 0;
@@ -1342,9 +1238,10 @@ SmemPlan plan_smem_f32(int n_bins, int n_geoms, int n_cells, int per_bin, size_t
     S.grad_in_smem = 1;
     used += (size_t)n_bins * 8;
   }
-  if (tail_threads > 0 && n_bins <= kOneBlockBins && used + (size_t)tail_threads * sizeof(Draw32) <= budget) {
+  const size_t slots = (size_t)(tail_threads / 32) * kTailSlots * sizeof(DrawLean);
+  if (tail_threads > 0 && n_bins <= kOneBlockBins && used + slots <= budget) {
     S.tail_slots = 1;
-    used += (size_t)tail_threads * sizeof(Draw32);
+    used += slots;
   }
   if (snap_threads > 0 && used + (size_t)snap_threads * 4 * sizeof(int4) <= budget) {
     S.snap_in_smem = 1;
