@@ -6,9 +6,9 @@
 // from event to event, and the event itself holds the geometry only.  Every
 // value is the event step's own (step_steady, apply_event) bit for bit.
 // Cycles per event of a lone particle (gray, 1 mm free path; 2.07 GHz), before
-// and now: 10 nm film 520 -> 286, pore lattice 771 -> 571, its measure-valued
-// gradient 1472 -> 1010 and likelihood-ratio gradient 1017 -> 587, square-pore
-// mesh 1379 -> 926.
+// and now: 10 nm film 520 -> 198 (half specular walls 520 -> 212), pore lattice
+// 771 -> 462, its measure-valued gradient 1472 -> 843 and likelihood-ratio
+// gradient 1017 -> 482, square-pore mesh 1379 -> 767.
 #pragma once
 
 #include "tracer.cuh"
@@ -27,15 +27,40 @@ struct __align__(16) DrawLean : Draw32 {
   uint32_t spec;
   // films: the flight across from wall to wall of the Lambertian direction,
   // and its tally from the lower wall
-  long long cq;
+  alignas(16) float film[3];   // {lam[1], lam[2], lam[0]}: read as one word with seg
   float seg;
-  float pad;
+  long long cq;
+  float pad[2];
 };
-static_assert(sizeof(DrawLean) == 96, "six 16-byte words");
+static_assert(sizeof(DrawLean) == 112, "seven 16-byte words");
 
 // Draws a warp computes ahead at once: two per lane.  A round's fixed cost
 // (votes, the counters' shuffles, the timer) is shared by that many events.
 constexpr int kTailSlots = 64;
+
+// What the loops take of the run's parameters, by value.
+struct LoneArgs {
+  uint32_t max_events;
+  int n_scat_max;
+  int n_bins, imp;
+  const uint64_t* spec_thr;
+  const uint4* relax_tab;
+  const float4* binf;
+  uint32_t k0, k1;
+};
+
+__device__ __forceinline__ void load_bin_lone(Particle<float>& p, const float4* binf) {
+  const float4 b = binf[p.bin];
+  p.v = b.x;
+  p.inv_v = b.y;
+  p.lam = b.z;
+}
+// the two-phonon clock restarted (draw_d2)
+__device__ __forceinline__ float d2_lone(const LoneArgs& A, int bin, float E2) {
+  if (!A.imp) return Num<float>::inf();
+  const float lam2 = A.binf[bin].w;
+  return isinf(lam2) ? Num<float>::inf() : lam2 * E2;
+}
 
 // Reciprocal by the hardware's approximation.  a * rcp_hw(b) has the bits of
 // __fdividef(a, b) for every b in the normal range (2^33 random pairs over
@@ -61,6 +86,9 @@ __device__ __forceinline__ void film_flight(DrawLean& d, const GeoRun& g, int W,
   d.seg = d.lam[0] != 0.0f ? fmaxf(geo_L<float>(g, W) * d.rlam[0], 0.0f) : Num<float>::big();
   float u[3];
   put3_cyclic<float>(u, W, d.lam[0], d.lam[1], d.lam[2]);
+  d.film[0] = d.lam[1];
+  d.film[1] = d.lam[2];
+  d.film[2] = d.lam[0];
   d.cq = fx_lone((s * d.seg) * sel3(u, ta));
 }
 
@@ -149,13 +177,12 @@ struct LeanDir {
 // the particle's end, or ALIVE once the slots are used up.
 // `walls`: the geometry's internal walls, to a multiple of four.
 template <class Grad, class Tally, bool EXT, bool CELLS, bool PORE>
-__device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, const WallLean* walls, const MatView& M,
-                                          const float4* binf, const RunCfg& C, const Tally& T, Grad& gr,
-                                          const DrawLean* slot0, uint32_t e_last) {
+__device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, const WallLean* walls, const LoneArgs& A,
+                                          const Tally& T, Grad& gr, const DrawLean* slot0, uint32_t e_last) {
   __builtin_assume(__isShared(slot0));   // shared-memory loads, not generic ones (half the latency)
   __builtin_assume(__isShared(walls));
   const uint32_t e0 = p.e;
-  const uint32_t e_lim = e_last < C.max_events - 1u ? e_last : C.max_events - 1u;
+  const uint32_t e_lim = e_last < A.max_events - 1u ? e_last : A.max_events - 1u;
   LeanBox box;
   box.load(g);
   const float cx = g.cxf, cy = g.cyf, r2 = g.r2f;
@@ -169,7 +196,7 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
   const int n_inner = EXT ? g.n_inner : 0;
   const unsigned perbin = EXT ? ((unsigned)g.fbin | ((unsigned)g.sbin << 7)) : 0u;
   uint64_t bin_thr = 0;
-  if (EXT && perbin) bin_thr = M.spec_thr[p.bin];
+  if (EXT && perbin) bin_thr = A.spec_thr[p.bin];
 
   while (p.e < e_lim) {
     const DrawLean& d = slot0[p.e - e0];
@@ -228,12 +255,12 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
         p.d_rel = p.d_rel - seg;
       } else {
         ++p.n_relax;
-        if (C.n_scat_max > 0 && p.n_relax >= C.n_scat_max) return STEP_DONE;
+        if (A.n_scat_max > 0 && p.n_relax >= A.n_scat_max) return STEP_DONE;
         T.period_end(p);
         p.bin = d.bin;
         p.d_rel = d.d_new;
-        load_bin(p, M, binf);
-        if (EXT && perbin) bin_thr = M.spec_thr[p.bin];
+        load_bin_lone(p, A.binf);
+        if (EXT && perbin) bin_thr = A.spec_thr[p.bin];
         if (Grad::on) {
           rlam = rcp_hw(p.lam);
           gr.resampled(p.bin, T.X(p));
@@ -244,7 +271,7 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
         p.u[a] = d.iso[a];
         D.r[a] = d.riso[a];
       }
-      if constexpr (EXT) p.d2 = draw_d2(p, M, binf, 0u, 0u, DrawSlot{&d});
+      if constexpr (EXT) p.d2 = d2_lone(A, p.bin, d.E2);
     } else {
       p.d_rel = p.d_rel - seg;
       if constexpr (EXT) p.d2 = p.d2 - seg;
@@ -308,7 +335,7 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
     D.aim(box, p.u);
     a2 = __fmaf_rn(p.u[0], p.u[0], __fmul_rn(p.u[1], p.u[1]));
   }
-  return p.e + 1u >= C.max_events ? STEP_TRUNCATED : STEP_ALIVE;
+  return p.e + 1u >= A.max_events ? STEP_TRUNCATED : STEP_ALIVE;
 }
 
 // The tail loop of a film: a box without pore or walls whose flights run
@@ -321,8 +348,7 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
 // number, so the event that ends a flight may lie past the slots and then
 // takes its draws inline (the same bits).
 template <int W, class Tally>
-__device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, const MatView& M, const uint4* relax_tab,
-                                          const float4* binf, const RunCfg& C, uint32_t k0, uint32_t k1, const Tally& T,
+__device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, const LoneArgs& R, const Tally& T,
                                           const DrawLean* slot0, uint32_t e_last) {
   constexpr int A = (W + 1) % 3, B = (W + 2) % 3;   // along the film; put3_cyclic's order
   const uint32_t e0 = p.e;
@@ -343,45 +369,69 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
     cq = fx_lone((s * db) * sel3(p.u, T.ta));
   };
   aim();
-  // Flights from wall to wall that neither relax, cross a periodic face nor end
-  // in a specular reflection: one branch each, the next draws read ahead.  An
-  // unsigned comparison of the bits takes 0 <= x < L in one test.
+  // Flights from wall to wall that do not relax, in a loop of their own with
+  // the next draws read ahead.  An unsigned comparison of the bits takes
+  // 0 <= x < L in one test; a flight past one periodic face is folded here
+  // (x -+ L, the value fold_periodic gives clear of its quotient's roundings),
+  // a specular reflection keeps the flight's length and tally.
   const uint32_t iLA = __float_as_uint(LA), iLB = __float_as_uint(LB);
   const bool quick = !across && !iso_lo && !iso_hi;
-  const uint32_t e_lim = e_last < C.max_events - 1u ? e_last : C.max_events - 1u;
+  const uint32_t e_lim = e_last < R.max_events - 1u ? e_last : R.max_events - 1u;
   for (;;) {
     if (quick && db < Num<float>::big()) {
       uint32_t hi = up ? 1u << f_hi : 1u << f_lo;
       const uint32_t both = (1u << f_hi) ^ (1u << f_lo);
       uint32_t e = p.e;
-      float x = p.x[A], y = p.x[B], ua = p.u[A], ub = p.u[B], dr = p.d_rel;
-      const DrawLean* d = slot0 + (e - e0);
-      float xn = __fmaf_rn(db, ua, x), yn = __fmaf_rn(db, ub, y);
-      bool moved = false;
-      float l0 = 0.0f;
+      float x = p.x[A], y = p.x[B], ua = p.u[A], ub = p.u[B], l0 = fabsf(p.u[W]), dr = p.d_rel;
+      long long X = p.Xq;
+      bool full = false;   // the flight ahead starts at a wall
       while (e < e_lim) {
-        if (!(dr >= db && __float_as_uint(xn) < iLA && __float_as_uint(yn) < iLB && (d->spec & hi) == 0u &&
-              d->lam[0] != 0.0f))
-          break;
-        p.Xq += cq;
+        const DrawLean* d = slot0 + (e - e0);
+        float4 nx = *reinterpret_cast<const float4*>(&d->film);   // {lam[1], lam[2], lam[0], seg}
+        long long nq = d->cq;
+        uint32_t sp = d->spec;
+        float xn = __fmaf_rn(db, ua, x), yn = __fmaf_rn(db, ub, y);
+        if (dr < db) break;
+        uint32_t n = 0u;
+        if (!(__float_as_uint(xn) < iLA && __float_as_uint(yn) < iLB)) {
+          bool fold = true;
+          if (!(__float_as_uint(xn) < iLA)) {
+            const float r = xn + (xn < 0.0f ? LA : -LA);
+            fold = xn > -0.999f * LA && xn < 1.999f * LA && __float_as_uint(r) < iLA;
+            xn = r;
+            n = 1u;
+          }
+          if (!(__float_as_uint(yn) < iLB)) {
+            const float r = yn + (yn < 0.0f ? LB : -LB);
+            fold = fold && yn > -0.999f * LB && yn < 1.999f * LB && __float_as_uint(r) < iLB;
+            yn = r;
+            ++n;
+          }
+          if (!fold || e + n >= e_lim) break;
+          d += n;
+          nx = *reinterpret_cast<const float4*>(&d->film);
+          nq = d->cq;
+          sp = d->spec;
+        }
+        const bool spec = (sp & hi) != 0u;
+        if (spec && !full) break;
+        X += cq;
         dr = dr - db;
         x = xn;
         y = yn;
-        db = d->seg;
-        cq = d->cq;
-        ua = d->lam[1];
-        ub = d->lam[2];
-        l0 = d->lam[0];
-        xn = __fmaf_rn(db, ua, x);
-        yn = __fmaf_rn(db, ub, y);
+        ua = spec ? ua : nx.x;
+        ub = spec ? ub : nx.y;
+        l0 = spec ? l0 : nx.z;
+        db = spec ? db : nx.w;
+        cq = spec ? cq : nq;
         hi ^= both;
-        moved = true;
-        ++e;
-        ++d;
+        full = true;
+        e += n + 1u;
       }
-      if (moved) {
+      if (full) {
         up = hi == 1u << f_hi;
         p.e = e;
+        p.Xq = X;
         p.d_rel = dr;
         p.x[A] = x;
         p.x[B] = y;
@@ -392,7 +442,7 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
         if (e >= e_last) return STEP_ALIVE;
       }
     }
-    if (p.e + 1u >= C.max_events) return STEP_TRUNCATED;
+    if (p.e + 1u >= R.max_events) return STEP_TRUNCATED;
     const bool relax = p.d_rel < db;
     const float seg = relax ? p.d_rel : db;
     uint32_t n = 0u;
@@ -400,9 +450,9 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
     p.x[B] = __fmaf_rn(seg, p.u[B], p.x[B]);
     if (!(p.x[A] >= 0.0f && p.x[A] < LA && p.x[B] >= 0.0f && p.x[B] < LB)) {
       n = fold_periodic(p.x, g.Lf, (1u << A) | (1u << B));
-      if (n >= C.max_events - 1u - p.e) {
+      if (n >= R.max_events - 1u - p.e) {
         p.Xq += relax ? fx_lone((s * seg) * sel3(p.u, T.ta)) : cq;
-        p.e = C.max_events - 1u;
+        p.e = R.max_events - 1u;
         return STEP_TRUNCATED;
       }
     }
@@ -413,21 +463,21 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
       p.Xq += fx_lone((s * seg) * sel3(p.u, T.ta));
       p.x[W] = __fmaf_rn(seg, p.u[W], p.x[W]);
       ++p.n_relax;
-      if (C.n_scat_max > 0 && p.n_relax >= C.n_scat_max) return STEP_DONE;
+      if (R.n_scat_max > 0 && p.n_relax >= R.n_scat_max) return STEP_DONE;
       T.period_end(p);
       if (si < nslots) {
         p.bin = d->bin;
         p.d_rel = d->d_new;
 #pragma unroll
         for (int a = 0; a < 3; ++a) p.u[a] = d->iso[a];
-        load_bin(p, M, binf);
+        load_bin_lone(p, R.binf);
       } else {
         Draw32 f;
-        draw_words(f, philox(make_uint4(p.pid, (uint32_t)p.g, p.e, 0u), k0, k1), relax_tab, M.n);
+        draw_words(f, philox(make_uint4(p.pid, (uint32_t)p.g, p.e, 0u), R.k0, R.k1), R.relax_tab, R.n_bins);
         p.bin = f.bin;
 #pragma unroll
         for (int a = 0; a < 3; ++a) p.u[a] = f.iso[a];
-        load_bin(p, M, binf);
+        load_bin_lone(p, R.binf);
         p.d_rel = p.lam * f.E;
       }
       aim();
@@ -447,11 +497,11 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
           p.u[B] = d->lam[2];
           db = d->seg;
           cq = up && across ? -d->cq : d->cq;
-          up = !up && p.u[W] != 0.0f;   // (lam[0] > 0)
+          up = !up;   // (lam[0] >= 2^-12)
         }
       } else {
         Draw32 f;
-        draw_words(f, philox(make_uint4(p.pid, (uint32_t)p.g, p.e, 0u), k0, k1), relax_tab, M.n);
+        draw_words(f, philox(make_uint4(p.pid, (uint32_t)p.g, p.e, 0u), R.k0, R.k1), R.relax_tab, R.n_bins);
         if ((uint64_t)f.wx < g.pthr[up ? f_hi : f_lo]) {
           p.u[W] = -p.u[W];
         } else {
@@ -464,6 +514,54 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
     }
     if (p.e >= e_last) return STEP_ALIVE;
   }
+}
+
+// A round of a particle's events by one of the loops.  Each is out of line, on
+// copies of the particle, the tally and the estimator: inlined into the tail
+// kernel the same loops ran longer (pore lattice 571 cycles an event, 462 out
+// of line and 344 alone in a small kernel), their instructions spread over a
+// kernel that a lone warp then fetches line by line.
+// LOOP: 0-2 a film across that axis, 3 a box, 4 a box with a pore.
+template <int LOOP, class Grad, class Tally, bool EXT, bool CELLS>
+static __device__ __noinline__ int trace_round(Particle<float>* pp, const GeoRun* g, const WallLean* walls, LoneArgs A,
+                                               const Tally* tt, Grad* gg, const DrawLean* slot0, uint32_t e_last) {
+  Particle<float> p = *pp;
+  const Tally T = *tt;
+  Grad gr = *gg;
+  int out;
+  if constexpr (LOOP < 3) out = trace_film<LOOP>(p, *g, A, T, slot0, e_last);
+  else out = trace_lean<Grad, Tally, EXT, CELLS, LOOP == 4>(p, *g, walls, A, T, gr, slot0, e_last);
+  *pp = p;
+  if (Grad::on) *gg = gr;
+  return out;
+}
+
+// The loop of the particle's geometry; `um`: the unfolded periodic axes where
+// they are a film's two, else 0.
+template <class Grad, class Tally, bool EXT, bool CELLS>
+__device__ __forceinline__ int trace_alone(Particle<float>& p, const GeoRun& g, const WallLean* walls, const LoneArgs& A,
+                                           const Tally& T, Grad& gr, const DrawLean* slot0, uint32_t e_last,
+                                           unsigned um) {
+  Particle<float> q = p;
+  const Tally Tq = T;
+  Grad gq = gr;
+  int out = STEP_ALIVE;
+#define MCBTE_LOOP(k) out = trace_round<k, Grad, Tally, EXT, CELLS>(&q, &g, walls, A, &Tq, &gq, slot0, e_last)
+  bool film = false;
+  if constexpr (!CELLS && !EXT && !Grad::on) {
+    film = um != 0u;
+    if (um == 3u) MCBTE_LOOP(2);
+    else if (um == 5u) MCBTE_LOOP(1);
+    else if (um == 6u) MCBTE_LOOP(0);
+  }
+  if (!film) {
+    if (g.pore) MCBTE_LOOP(4);
+    else MCBTE_LOOP(3);
+  }
+#undef MCBTE_LOOP
+  p = q;
+  if (Grad::on) gr = gq;
+  return out;
 }
 
 }  // namespace mcbte

@@ -741,10 +741,14 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
       } else {
         // log2 of the slots per particle: nlive << sh <= kTailSlots
         const int sh = (kTailSlots == 64 ? 6 : 5) - (32 - __clz(nlive - 1));
-        for (unsigned i = lane; i < (unsigned)kTailSlots; i += 32u) {
+#pragma unroll
+        for (int h = 0; h < kTailSlots / 32; ++h) {
+          const unsigned i = lane + 32u * h;
           const int r = (int)(i >> sh);   // the live particle slot i belongs to
+          // its lane: a lone particle's is the only one, else the r-th live lane
           unsigned mm = live;
-          for (int k = 0; k < r && mm; ++k) mm &= mm - 1u;
+          if (nlive > 1)
+            for (int k = 0; k < r && mm; ++k) mm &= mm - 1u;
           const int owner = mm ? __ffs(mm) - 1 : 0;
           const uint32_t e_o = __shfl_sync(kAll, p.e, owner);
           const uint32_t pid_o = __shfl_sync(kAll, p.pid, owner);
@@ -781,20 +785,15 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
           const DrawLean* s0 = slots + (__popc(live & ((1u << lane) - 1u)) << sh);
           const unsigned um = UNF ? unfold_mask<GradT>(*G, C) : 0u;
           const uint32_t e_f = p.e, e_l = p.e + (1u << sh);
-          if (UNF && um == 3u)
-            out = trace_film<2>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l);
-          else if (UNF && um == 5u)
-            out = trace_film<1>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l);
-          else if (UNF && um == 6u)
-            out = trace_film<0>(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l);
-          else if (UNF && um)
+          const bool film = um == 3u || um == 5u || um == 6u;
+          if (UNF && um && !film) {
             out = trace_unfolded(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, um);
-          else if (EXT && (C.n_regs > 0 || C.nscat_acc || (C.n_geoms > 1 && G->n_inner > 0)))
+          } else if (EXT && (C.n_regs > 0 || C.nscat_acc || (C.n_geoms > 1 && G->n_inner > 0))) {
             out = trace_slots<GradT, decltype(T)>(p, *G, M, relax, binf, C, key.x, key.y, T, gr, s0, e_l);
-          else if (G->pore)
-            out = trace_lean<GradT, decltype(T), EXT, (CELLS > 0), true>(p, *G, s_walls, M, binf, C, T, gr, s0, e_l);
-          else
-            out = trace_lean<GradT, decltype(T), EXT, (CELLS > 0), false>(p, *G, s_walls, M, binf, C, T, gr, s0, e_l);
+          } else {
+            const LoneArgs la{C.max_events, C.n_scat_max, n, M.imp, M.spec_thr, relax, binf, key.x, key.y};
+            out = trace_alone<GradT, decltype(T), EXT, (CELLS > 0)>(p, *G, s_walls, la, T, gr, s0, e_l, um);
+          }
           // (the time budget every 256 events)
           if (out == STEP_ALIVE && ((e_f ^ p.e) >> 8) != 0u && globaltimer_ns() > deadline) {
             atomicOr(A.flags, 1);
