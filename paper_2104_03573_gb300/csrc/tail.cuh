@@ -6,9 +6,9 @@
 // from event to event, and the event itself holds the geometry only.  Every
 // value is the event step's own (step_steady, apply_event) bit for bit.
 // Cycles per event of a lone particle (gray, 1 mm free path; 2.07 GHz), before
-// and now: 10 nm film 520 -> 198 (half specular walls 520 -> 212), pore lattice
-// 771 -> 462, its measure-valued gradient 1472 -> 843 and likelihood-ratio
-// gradient 1017 -> 482, square-pore mesh 1379 -> 767.
+// and now: 10 nm film 520 -> 194 (half specular walls 520 -> 208), pore lattice
+// 771 -> 451, its measure-valued gradient 1472 -> 841 and likelihood-ratio
+// gradient 1017 -> 483, square-pore mesh 1379 -> 767.
 #pragma once
 
 #include "tracer.cuh"
@@ -19,20 +19,25 @@ namespace mcbte {
 // draws of Draw32, the reciprocals of both directions' components (0 where a
 // component is 0), the relaxation's new distance, and the specular test
 // against every surface of the geometry (bits 0-5 faces, 6 the pore, 7 + k
-// wall k).
+// wall k).  80 bytes, so that a gradient's slots leave room for its pore-hit
+// snapshots; a film (trace_film) needs no reciprocals and keeps in their place
+// {lam[1], lam[2], lam[0], the length of the flight across} and {its tally from
+// the lower wall (64 bits), the relaxation's distance}.
 struct __align__(16) DrawLean : Draw32 {
   float riso[3];
   float d_new;
   float rlam[3];
   uint32_t spec;
-  // films: the flight across from wall to wall of the Lambertian direction,
-  // and its tally from the lower wall
-  alignas(16) float film[3];   // {lam[1], lam[2], lam[0]}: read as one word with seg
-  float seg;
-  long long cq;
-  float pad[2];
+
+  __device__ __forceinline__ float4 film_flight() const { return make_float4(riso[0], riso[1], riso[2], d_new); }
+  __device__ __forceinline__ long long film_tally() const {
+    return (long long)(((unsigned long long)__float_as_uint(rlam[1]) << 32) | __float_as_uint(rlam[0]));
+  }
+  __device__ __forceinline__ float film_d_new() const { return rlam[2]; }
+  // W: the film's wall axis; s: the particle's sign
+  __device__ __forceinline__ void to_film(float LW, int W, float s, int ta);
 };
-static_assert(sizeof(DrawLean) == 112, "seven 16-byte words");
+static_assert(sizeof(DrawLean) == 80, "five 16-byte words");
 
 // Draws a warp computes ahead at once: two per lane.  A round's fixed cost
 // (votes, the counters' shuffles, the timer) is shared by that many events.
@@ -81,15 +86,18 @@ __device__ __forceinline__ long long fx_lone(float contrib) {
   return fabsf(s) < 2.0e9f ? (long long)__float2int_rn(s) : __float2ll_rn(s);
 }
 
-// W: the wall axis of a film (trace_film); s: the particle's sign.
-__device__ __forceinline__ void film_flight(DrawLean& d, const GeoRun& g, int W, float s, int ta) {
-  d.seg = d.lam[0] != 0.0f ? fmaxf(geo_L<float>(g, W) * d.rlam[0], 0.0f) : Num<float>::big();
+__device__ __forceinline__ void DrawLean::to_film(float LW, int W, float s, int ta) {
+  const float seg = lam[0] != 0.0f ? fmaxf(LW * rlam[0], 0.0f) : Num<float>::big();
   float u[3];
-  put3_cyclic<float>(u, W, d.lam[0], d.lam[1], d.lam[2]);
-  d.film[0] = d.lam[1];
-  d.film[1] = d.lam[2];
-  d.film[2] = d.lam[0];
-  d.cq = fx_lone((s * d.seg) * sel3(u, ta));
+  put3_cyclic<float>(u, W, lam[0], lam[1], lam[2]);
+  const unsigned long long q = (unsigned long long)fx_lone((s * seg) * sel3(u, ta));
+  rlam[2] = d_new;
+  rlam[0] = __uint_as_float((uint32_t)q);
+  rlam[1] = __uint_as_float((uint32_t)(q >> 32));
+  riso[0] = lam[1];
+  riso[1] = lam[2];
+  riso[2] = lam[0];
+  d_new = seg;
 }
 
 __device__ __forceinline__ void draw_lean(DrawLean& d, const GeoRun& g, const float4* binf, bool ext) {
@@ -387,8 +395,8 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
       bool full = false;   // the flight ahead starts at a wall
       while (e < e_lim) {
         const DrawLean* d = slot0 + (e - e0);
-        float4 nx = *reinterpret_cast<const float4*>(&d->film);   // {lam[1], lam[2], lam[0], seg}
-        long long nq = d->cq;
+        float4 nx = d->film_flight();
+        long long nq = d->film_tally();
         uint32_t sp = d->spec;
         float xn = __fmaf_rn(db, ua, x), yn = __fmaf_rn(db, ub, y);
         if (dr < db) break;
@@ -409,8 +417,8 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
           }
           if (!fold || e + n >= e_lim) break;
           d += n;
-          nx = *reinterpret_cast<const float4*>(&d->film);
-          nq = d->cq;
+          nx = d->film_flight();
+          nq = d->film_tally();
           sp = d->spec;
         }
         const bool spec = (sp & hi) != 0u;
@@ -467,7 +475,7 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
       T.period_end(p);
       if (si < nslots) {
         p.bin = d->bin;
-        p.d_rel = d->d_new;
+        p.d_rel = d->film_d_new();
 #pragma unroll
         for (int a = 0; a < 3; ++a) p.u[a] = d->iso[a];
         load_bin_lone(p, R.binf);
@@ -495,8 +503,8 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
           p.u[W] = up ? -d->lam[0] : d->lam[0];
           p.u[A] = d->lam[1];
           p.u[B] = d->lam[2];
-          db = d->seg;
-          cq = up && across ? -d->cq : d->cq;
+          db = d->d_new;
+          cq = up && across ? -d->film_tally() : d->film_tally();
           up = !up;   // (lam[0] >= 2^-12)
         }
       } else {
@@ -518,7 +526,7 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
 
 // A round of a particle's events by one of the loops.  Each is out of line, on
 // copies of the particle, the tally and the estimator: inlined into the tail
-// kernel the same loops ran longer (pore lattice 571 cycles an event, 462 out
+// kernel the same loops ran longer (pore lattice 571 cycles an event, 451 out
 // of line and 344 alone in a small kernel), their instructions spread over a
 // kernel that a lone warp then fetches line by line.
 // LOOP: 0-2 a film across that axis, 3 a box, 4 a box with a pore.

@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
             if constexpr (UNF) {
               const unsigned um_o = unfold_mask<GradT>(geos[g_o], C);
               const int W = um_o == 3u ? 2 : (um_o == 5u ? 1 : (um_o == 6u ? 0 : -1));
-              if (W >= 0) film_flight(d, geos[g_o], W, s_o, T.ta);
+              if (W >= 0) d.to_film(geo_L<float>(geos[g_o], W), W, s_o, T.ta);
             }
             slots[i] = d;
           }
