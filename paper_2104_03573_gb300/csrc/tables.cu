@@ -52,15 +52,39 @@ __global__ void k_bins(MatBuild b) {
 // sums block stages three weight columns).
 constexpr int kAliasSmemBins = 9216;
 
+// Sum of w[0..n) in index order.  The chain of additions is the sum's time (an
+// FP64 addition takes some 60 cycles here); the reads run ahead of it.
+__device__ __forceinline__ double ordered_sum(const double* w, int n) {
+  double s = 0.0;
+  int i = 0;
+  for (; i + 8 <= n; i += 8) {
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = w[i + j];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s += v[j];
+  }
+  for (; i < n; ++i) s += w[i];
+  return s;
+}
+
+// x < 1 for x >= 0, by the bits (a comparison of the FP64 pipe waits as long
+// as an addition)
+__device__ __forceinline__ bool below_one(double x) { return __double_as_longlong(x) < 0x3ff0000000000000ll; }
+
 // blockIdx.x = 0..2 builds alias table k (weights C v, C, C / tau);
-// blockIdx.x = 3 forms the sums and the relaxation pmf.  The sums and
-// Vose's lists are sequential (thread 0, bin order, so the table is a fixed
-// function of the weights); the per-bin arithmetic around them is spread
-// over the block.  With `smem` the work arrays live in shared memory, else
-// in the global scratch.
+// blockIdx.x = 3 forms the sums and the relaxation pmf.  The sums and the
+// walk through Vose's lists are sequential (bin order, so the table is a fixed
+// function of the weights), and their dependent FP64 additions are the
+// kernel's time: one per bin for a sum (the three sums on three warps), two
+// per bin for the walk, which keeps the bin it fills in registers and reads
+// the next ones ahead.  The lists and the per-bin arithmetic are the block's.
+// With `smem` the work arrays live in shared memory, else in the global
+// scratch.  3000 bins: 774 us with the lists and the walk read step by step.
 __global__ void k_alias(MatBuild b, int smem) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ double s_tot;
+  __shared__ int s_cnt[8];
   const int n = b.n;
   const int k = blockIdx.x;
   const int t = threadIdx.x;
@@ -80,15 +104,10 @@ __global__ void k_alias(MatBuild b, int smem) {
       c1 = st + n;
       c2 = st + 2 * (size_t)n;
     }
-    if (t == 0) {
-      double ct = 0.0, cv = 0.0, cr = 0.0;
-      for (int i = 0; i < n; ++i) {
-        ct += c0[i];
-        cv += c1[i];
-        cr += c2[i];
-      }
-      b.sums[0] = ct;
-      b.sums[1] = cv;
+    if (t == 0) b.sums[0] = ordered_sum(c0, n);
+    if (t == 32) b.sums[1] = ordered_sum(c1, n);
+    if (t == 64) {
+      const double cr = ordered_sum(c2, n);
       b.sums[2] = cr;
       s_tot = cr;
     }
@@ -113,11 +132,7 @@ __global__ void k_alias(MatBuild b, int smem) {
   }
   for (int i = t; i < n; i += blockDim.x) p[i] = w[i];
   __syncthreads();
-  if (t == 0) {
-    double W = 0.0;
-    for (int i = 0; i < n; ++i) W += p[i];
-    s_tot = W;
-  }
+  if (t == 0) s_tot = ordered_sum(p, n);
   __syncthreads();
   const double W = s_tot;
   for (int i = t; i < n; i += blockDim.x) {
@@ -125,20 +140,69 @@ __global__ void k_alias(MatBuild b, int smem) {
     alias[i] = i;
   }
   __syncthreads();
-  if (t == 0) {
-    int ns = 0, nl = 0;
-    for (int i = 0; i < n; ++i) {
-      if (p[i] < 1.0) small[ns++] = i; else large[nl++] = i;
-    }
-    // a bin popped from the small list keeps its p as its probability and
-    // takes the large bin as its alias (never itself); every other bin
-    // keeps probability 1
-    while (ns > 0 && nl > 0) {
-      const int l = small[--ns];
-      const int g = large[--nl];
+  // the lists in bin order: each thread a run of bins, placed by the number of
+  // small ones before it
+  const int per = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+  const int i0 = min(t * per, n), i1 = min(i0 + per, n);
+  int mine = 0;
+  for (int i = i0; i < i1; ++i) mine += p[i] < 1.0 ? 1 : 0;
+  int at = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, at, o);
+    if ((t & 31) >= o) at += y;
+  }
+  if ((t & 31) == 31) s_cnt[t >> 5] = at;
+  __syncthreads();
+  int ns = 0;
+  for (int q = 0; q < 8; ++q) {
+    if (q < (t >> 5)) at += s_cnt[q];
+    ns += s_cnt[q];
+  }
+  int si = at - mine, li = i0 - si;
+  for (int i = i0; i < i1; ++i) {
+    if (p[i] < 1.0) small[si++] = i; else large[li++] = i;
+  }
+  __syncthreads();
+  int nl = n - ns;
+  if (t == 0 && ns > 0 && nl > 0) {
+    // Vose's walk: pop a small bin l and a large one g, l's alias is g and g
+    // gives up 1 - p[l]; g returns to the list it now belongs to and is popped
+    // from there at once, so it stays in registers until it is small and has
+    // its own alias (a bin popped from the small list keeps its p as its
+    // probability and takes the large bin as its alias, never itself; every
+    // other bin keeps probability 1).
+    int g = large[--nl];
+    double pg = p[g];
+    int l = small[--ns];
+    double pl = p[l];
+    int gn = nl > 0 ? large[nl - 1] : 0, ln = ns > 0 ? small[ns - 1] : 0;   // the next ones
+    double pgn = p[gn], pln = p[ln];
+    for (;;) {
       alias[l] = g;
-      p[g] = (p[g] + p[l]) - 1.0;
-      if (p[g] < 1.0) small[ns++] = g; else large[nl++] = g;
+      pg = (pg + pl) - 1.0;
+      if (below_one(pg)) {
+        // g is the next small bin
+        p[g] = pg;
+        if (nl == 0) break;
+        l = g;
+        pl = pg;
+        g = gn;
+        pg = pgn;
+        --nl;
+        gn = nl > 0 ? large[nl - 1] : 0;
+        pgn = p[gn];
+      } else {
+        if (ns == 0) {
+          p[g] = pg;
+          break;
+        }
+        l = ln;
+        pl = pln;
+        --ns;
+        ln = ns > 0 ? small[ns - 1] : 0;
+        pln = p[ln];
+      }
     }
   }
   __syncthreads();
