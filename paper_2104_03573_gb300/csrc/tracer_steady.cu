@@ -1124,7 +1124,7 @@ cudaError_t launch_f64(const GeoRun* geos, const uint64_t* offs, const MatView& 
   auto kern = k_steady_fp64<CELLS, GRAD>;
   const int blocks = f64_blocks(C.total);
   RunCfg R = C;
-  R.take_chunk = take_chunk(C.total, (uint64_t)blocks * (kF64Threads / 32), 256u);
+  R.take_chunk = take_chunk(C.total, (uint64_t)blocks * (kF64Threads / 32), 256u, (uint64_t)blocks * 4, 1u);
   kern<<<blocks, kF64Threads, 0, s>>>(geos, offs, M, R, A);
   return cudaGetLastError();
 }
@@ -1150,7 +1150,8 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
   if (occ < 1) return cudaErrorInvalidConfiguration;
   const int b = (bps > 0 && bps < occ) ? bps : occ;
   RunCfg R = C;
-  R.take_chunk = take_chunk(C.total, (uint64_t)sm_count() * b * (TPB / 32), C.take_chunk);
+  const uint64_t warps = (uint64_t)sm_count() * b * (TPB / 32);
+  R.take_chunk = take_chunk(C.total, warps, C.take_chunk, warps, MODE == 0 ? 4u : 16u);
   kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, offs, M, R, A, S);
   return cudaGetLastError();
 }

@@ -678,7 +678,7 @@ cudaError_t launch_transient(int precision, const GeoRun* geos, const MatView& M
   if (precision == MCBTE_FP64_PLAIN) {
     const int blocks = f64_blocks(C.total);
     RunCfg R = C;
-    R.take_chunk = take_chunk(C.total, (uint64_t)blocks * (kF64Threads / 32), 256u);
+    R.take_chunk = take_chunk(C.total, (uint64_t)blocks * (kF64Threads / 32), 256u, (uint64_t)blocks * 4, 1u);
     k_transient_fp64<<<blocks, kF64Threads, 0, s>>>(geos, M, R, A);
     return cudaGetLastError();
   }
@@ -704,7 +704,8 @@ cudaError_t launch_transient_tav(const GeoRun* geos, const MatView& M, const Run
   if (occ < 1) return cudaErrorInvalidConfiguration;
   const int b = (bps > 0 && bps < occ) ? bps : occ;
   RunCfg R = C;
-  R.take_chunk = take_chunk(C.total, (uint64_t)sm_count() * b * (TPB / 32), C.take_chunk);
+  const uint64_t warps = (uint64_t)sm_count() * b * (TPB / 32);
+  R.take_chunk = take_chunk(C.total, warps, C.take_chunk, warps, 4u);
   kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, M, R, A, S);
   return cudaGetLastError();
 }
