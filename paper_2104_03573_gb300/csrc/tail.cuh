@@ -346,6 +346,20 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
   return p.e + 1u >= A.max_events ? STEP_TRUNCATED : STEP_ALIVE;
 }
 
+// Events per flight of a film's particle: a diffuse flight across it meets
+// LW / LA + LW / LB periodic faces in the mean, each of them an event number
+// (and a draw computed ahead that nothing reads).  0: not a film.
+__device__ __forceinline__ float film_events(const GeoRun& g, unsigned um) {
+  const int W = um == 3u ? 2 : (um == 5u ? 1 : (um == 6u ? 0 : -1));
+  if (W < 0) return 0.0f;
+  const float LW = geo_L<float>(g, W), LA = geo_L<float>(g, (W + 1) % 3), LB = geo_L<float>(g, (W + 2) % 3);
+  return 1.0f + LW * rcp_hw(LA) + LW * rcp_hw(LB);
+}
+// A round of draws ahead costs a warp about as much as four flights that draw
+// inline, so thick films, whose slots end before that, take no slots.
+constexpr float kInlineFlights = 4.0f;
+constexpr float kInlineRound = 32.0f;   // flights of a round without slots (then the warp votes again)
+
 // The tail loop of a film: a box without pore or walls whose flights run
 // through the two periodic axes (forward run without cell tallies or extended
 // physics), so that the faces left are the pair across axis W.  A flight from
@@ -354,13 +368,13 @@ __device__ __forceinline__ int trace_lean(Particle<float>& p, const GeoRun& g, c
 // from flight to flight holds two additions along the film, the relaxation
 // clock and the fold at the periodic faces.  The crossings advance the event
 // number, so the event that ends a flight may lie past the slots and then
-// takes its draws inline (the same bits).
+// takes its draws inline (the same bits).  nslots: the draws at slot0, or 0 to
+// take every event's inline up to event e_last.
 template <int W, class Tally>
 __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, const LoneArgs& R, const Tally& T,
-                                          const DrawLean* slot0, uint32_t e_last) {
+                                          const DrawLean* slot0, uint32_t nslots, uint32_t e_last) {
   constexpr int A = (W + 1) % 3, B = (W + 2) % 3;   // along the film; put3_cyclic's order
   const uint32_t e0 = p.e;
-  const uint32_t nslots = e_last - e0;
   const float LA = g.Lf[A], LB = g.Lf[B], LW = g.Lf[W];
   const int f_lo = axis_min_face(W), f_hi = axis_max_face(W);
   const bool iso_lo = g.type[f_lo] == MCBTE_FACE_ISOTHERMAL, iso_hi = g.type[f_hi] == MCBTE_FACE_ISOTHERMAL;
@@ -383,7 +397,7 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
   // (x -+ L, the value fold_periodic gives clear of its quotient's roundings),
   // a specular reflection keeps the flight's length and tally.
   const uint32_t iLA = __float_as_uint(LA), iLB = __float_as_uint(LB);
-  const bool quick = !across && !iso_lo && !iso_hi;
+  const bool quick = nslots != 0u && !across && !iso_lo && !iso_hi;
   const uint32_t e_lim = e_last < R.max_events - 1u ? e_last : R.max_events - 1u;
   for (;;) {
     if (quick && db < Num<float>::big()) {
@@ -415,7 +429,17 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
             yn = r;
             ++n;
           }
-          if (!fold || e + n >= e_lim) break;
+          if (!fold) {
+            // past more than one period (films thicker than their period)
+            float q[3];
+            q[W] = 0.0f;
+            q[A] = __fmaf_rn(db, ua, x);
+            q[B] = __fmaf_rn(db, ub, y);
+            n = fold_periodic(q, g.Lf, (1u << A) | (1u << B));
+            xn = q[A];
+            yn = q[B];
+          }
+          if (n >= e_lim - e) break;
           d += n;
           nx = d->film_flight();
           nq = d->film_tally();
@@ -532,12 +556,13 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
 // LOOP: 0-2 a film across that axis, 3 a box, 4 a box with a pore.
 template <int LOOP, class Grad, class Tally, bool EXT, bool CELLS>
 static __device__ __noinline__ int trace_round(Particle<float>* pp, const GeoRun* g, const WallLean* walls, LoneArgs A,
-                                               const Tally* tt, Grad* gg, const DrawLean* slot0, uint32_t e_last) {
+                                               const Tally* tt, Grad* gg, const DrawLean* slot0, uint32_t nslots,
+                                               uint32_t e_last) {
   Particle<float> p = *pp;
   const Tally T = *tt;
   Grad gr = *gg;
   int out;
-  if constexpr (LOOP < 3) out = trace_film<LOOP>(p, *g, A, T, slot0, e_last);
+  if constexpr (LOOP < 3) out = trace_film<LOOP>(p, *g, A, T, slot0, nslots, e_last);
   else out = trace_lean<Grad, Tally, EXT, CELLS, LOOP == 4>(p, *g, walls, A, T, gr, slot0, e_last);
   *pp = p;
   if (Grad::on) *gg = gr;
@@ -548,13 +573,13 @@ static __device__ __noinline__ int trace_round(Particle<float>* pp, const GeoRun
 // they are a film's two, else 0.
 template <class Grad, class Tally, bool EXT, bool CELLS>
 __device__ __forceinline__ int trace_alone(Particle<float>& p, const GeoRun& g, const WallLean* walls, const LoneArgs& A,
-                                           const Tally& T, Grad& gr, const DrawLean* slot0, uint32_t e_last,
-                                           unsigned um) {
+                                           const Tally& T, Grad& gr, const DrawLean* slot0, uint32_t nslots,
+                                           uint32_t e_last, unsigned um) {
   Particle<float> q = p;
   const Tally Tq = T;
   Grad gq = gr;
   int out = STEP_ALIVE;
-#define MCBTE_LOOP(k) out = trace_round<k, Grad, Tally, EXT, CELLS>(&q, &g, walls, A, &Tq, &gq, slot0, e_last)
+#define MCBTE_LOOP(k) out = trace_round<k, Grad, Tally, EXT, CELLS>(&q, &g, walls, A, &Tq, &gq, slot0, nslots, e_last)
   bool film = false;
   if constexpr (!CELLS && !EXT && !Grad::on) {
     film = um != 0u;

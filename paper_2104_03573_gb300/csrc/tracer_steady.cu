@@ -741,8 +741,18 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
       } else {
         // log2 of the slots per particle: nlive << sh <= kTailSlots
         const int sh = (kTailSlots == 64 ? 6 : 5) - (32 - __clz(nlive - 1));
+        const unsigned um = (UNF && alive) ? unfold_mask<GradT>(*G, C) : 0u;
+        // draws ahead, or (most of the live particles in thick films) inline
+        bool ahead = true;
+        float per_flight = 0.0f;
+        if constexpr (UNF) {
+          if (alive) per_flight = film_events(*G, um);
+          const bool inl = per_flight * kInlineFlights > (float)(1u << sh);
+          ahead = 2 * __popc(__ballot_sync(kAll, alive && inl)) <= nlive || __any_sync(kAll, alive && per_flight == 0.0f);
+        }
 #pragma unroll
         for (int h = 0; h < kTailSlots / 32; ++h) {
+          if (!ahead) break;
           const unsigned i = lane + 32u * h;
           const int r = (int)(i >> sh);   // the live particle slot i belongs to
           // its lane: a lone particle's is the only one, else the r-th live lane
@@ -783,8 +793,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
         __syncwarp();
         if (alive) {
           const DrawLean* s0 = slots + (__popc(live & ((1u << lane) - 1u)) << sh);
-          const unsigned um = UNF ? unfold_mask<GradT>(*G, C) : 0u;
-          const uint32_t e_f = p.e, e_l = p.e + (1u << sh);
+          const uint32_t e_f = p.e, nslots = ahead ? 1u << sh : 0u, e_l = p.e + (ahead ? nslots : (uint32_t)fminf(kInlineRound * per_flight, 65536.0f));
           const bool film = um == 3u || um == 5u || um == 6u;
           if (UNF && um && !film) {
             out = trace_unfolded(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, um);
@@ -792,7 +801,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
             out = trace_slots<GradT, decltype(T)>(p, *G, M, relax, binf, C, key.x, key.y, T, gr, s0, e_l);
           } else {
             const LoneArgs la{C.max_events, C.n_scat_max, n, M.imp, M.spec_thr, relax, binf, key.x, key.y};
-            out = trace_alone<GradT, decltype(T), EXT, (CELLS > 0)>(p, *G, s_walls, la, T, gr, s0, e_l, um);
+            out = trace_alone<GradT, decltype(T), EXT, (CELLS > 0)>(p, *G, s_walls, la, T, gr, s0, nslots, e_l, um);
           }
           // (the time budget every 256 events)
           if (out == STEP_ALIVE && ((e_f ^ p.e) >> 8) != 0u && globaltimer_ns() > deadline) {

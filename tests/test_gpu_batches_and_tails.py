@@ -124,12 +124,12 @@ def test_snapshot_records_on_ragged_grids(n, grid, times, even):
     assert np.array_equal(a["tally"], b["tally"]) and np.array_equal(a["events_pp"], b["events_pp"])
 
 
-def _film_across(axis, p, wall):
+def _film_across(axis, p, wall, d):
     ft, fp, fT = [W.PERIODIC] * 6, [0.0] * 6, [0.0] * 6
     for f, dT in zip(FACES[axis], (0.5, -0.5)):
         ft[f], fp[f], fT[f] = wall, p, 300.0 + dT
     size, grad = [100e-9] * 3, [0.0] * 3
-    size[axis] = 20e-9 if wall == W.ADIABATIC else 400e-9
+    size[axis] = d
     tally = axis
     if wall == W.ADIABATIC:
         tally = (axis + 1) % 3
@@ -155,14 +155,16 @@ def _same_with_and_without_tail(mat, geo, n, tally, **kw):
 @pytest.mark.parametrize("axis", [0, 1, 2])
 @pytest.mark.parametrize("p", [0.0, 0.4, 1.0])
 @pytest.mark.parametrize("max_events", [10 ** 7, 777])
-def test_film_tails_along_every_axis(axis, p, max_events):
-    geo, tally = _film_across(axis, p, W.ADIABATIC)
+@pytest.mark.parametrize("d", [20e-9, 300e-9, 2000e-9])   # the period is 100 nm: few, several, many faces a flight
+def test_film_tails_along_every_axis(axis, p, max_events, d):
+    geo, tally = _film_across(axis, p, W.ADIABATIC, d)
     _same_with_and_without_tail(W.bvk_holland(), geo, 20_011, tally, max_events=max_events)
 
 
 @pytest.mark.parametrize("axis", [0, 1, 2])
-def test_wall_to_wall_tails_along_every_axis(axis):
-    geo, tally = _film_across(axis, 0.0, W.ISOTHERMAL)
+@pytest.mark.parametrize("d", [400e-9, 2000e-9])
+def test_wall_to_wall_tails_along_every_axis(axis, d):
+    geo, tally = _film_across(axis, 0.0, W.ISOTHERMAL, d)
     _same_with_and_without_tail(W.gray(6000.0, 5e-9), geo, 5003, tally)
 
 
