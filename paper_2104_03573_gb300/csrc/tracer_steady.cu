@@ -83,8 +83,6 @@ struct GradPick<false, On> { using type = GradOff; };
 // SX: the tally's type, 2^-20 nm whole numbers (FP32 path, exact) or FP64 nm.
 __device__ __forceinline__ double tally_nm(long long x) { return (double)x * kFxInv; }
 __device__ __forceinline__ double tally_nm(double x) { return x; }
-__device__ __forceinline__ void tally_add(long long* a, long long x) { red_s64(a, x); }
-__device__ __forceinline__ void tally_add(double* a, double x) { atomicAdd(a, x); }
 
 template <typename SX>
 struct ThreadAcct {
@@ -133,6 +131,39 @@ struct ThreadAcct {
   }
 };
 
+// The sum of the block's tallies.  A lane's sum fits 64 bits (2^43 nm), a
+// block's need not (gray, 30 m free path: 2e5 particles wrapped), so a block
+// adds the halves apart, the upper one signed; whole numbers, hence the same
+// sum in any order.
+template <typename SX> struct BlockSum;
+template <> struct BlockSum<long long> {
+  long long hi, lo;
+  __device__ __forceinline__ void reset() { hi = lo = 0; }
+  // x: this lane's; called by all 32 lanes, lane 0 adds
+  __device__ __forceinline__ void add(long long x) {
+    long long h = x >> 32, l = (long long)(unsigned)x;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      h += __shfl_xor_sync(0xffffffffu, h, o);
+      l += __shfl_xor_sync(0xffffffffu, l, o);
+    }
+    if ((threadIdx.x & 31u) != 0u) return;
+    red_s64(&hi, h);
+    red_s64(&lo, l);
+  }
+  __device__ __forceinline__ double nm() const { return ((double)hi * 4294967296.0 + (double)lo) * kFxInv; }
+};
+template <> struct BlockSum<double> {
+  double v;
+  __device__ __forceinline__ void reset() { v = 0.0; }
+  __device__ __forceinline__ void add(double x) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31u) == 0u) atomicAdd(&v, x);
+  }
+  __device__ __forceinline__ double nm() const { return v; }
+};
+
 // A block's book-keeping (shared memory), for runs of one geometry.  Every
 // lane of the grid flushing its own fields queued 8e5 atomics on seven
 // addresses (about 0.4 ms, whatever the run's length: a gray slab of 1e5
@@ -142,20 +173,19 @@ template <typename SX>
 struct BlockAcct {
   unsigned long long ev, trunc, maxev, traced;
   long long s_emit, s_abs, absorbed;
-  SX sx;
+  BlockSum<SX> sx;
   double sx2;
 
   __device__ __forceinline__ void reset() {
     ev = trunc = maxev = traced = 0ull;
     s_emit = s_abs = absorbed = 0;
-    sx = SX(0);
+    sx.reset();
     sx2 = 0.0;
   }
   // called by all 32 lanes of a warp
   __device__ __forceinline__ void add(const ThreadAcct<SX>& t) {
     constexpr unsigned kAll = 0xffffffffu;
     unsigned long long ev_w = t.ev;
-    SX sx_w = t.sx;
     long long se = t.s_emit, sa = t.s_abs;
     double s2 = t.sx2;
     unsigned long long tr = t.traced;
@@ -164,18 +194,18 @@ struct BlockAcct {
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) {
       ev_w += __shfl_xor_sync(kAll, ev_w, o);
-      sx_w += __shfl_xor_sync(kAll, sx_w, o);
       se += __shfl_xor_sync(kAll, se, o);
       sa += __shfl_xor_sync(kAll, sa, o);
       s2 += __shfl_xor_sync(kAll, s2, o);
       tr += __shfl_xor_sync(kAll, tr, o);
     }
-    if ((threadIdx.x & 31u) != 0u || tr == 0ull) return;
+    if (tr == 0ull) return;   // the same in every lane
+    sx.add(t.sx);
+    if ((threadIdx.x & 31u) != 0u) return;
     atomicAdd(&ev, ev_w);
     if (tc) atomicAdd(&trunc, (unsigned long long)tc);
     atomicMax(&maxev, (unsigned long long)mx);
     atomicAdd(&traced, tr);
-    tally_add(&sx, sx_w);
     atomicAdd(&sx2, s2);
     red_s64(&s_emit, se);
     if (ab) {
@@ -190,7 +220,7 @@ struct BlockAcct {
     if (trunc) atomicAdd(&A.cnt[1], trunc);
     atomicMax(&A.cnt[2], maxev);
     atomicAdd(&A.cnt[3], traced);
-    atomicAdd(&A.dsc[0], tally_nm(sx));
+    atomicAdd(&A.dsc[0], sx.nm());
     atomicAdd(&A.dsc[1], sx2);
     atomicAdd(&A.dsc[2], (double)s_emit);
     if (absorbed) {
