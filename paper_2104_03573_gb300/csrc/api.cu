@@ -705,6 +705,7 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
   C.refill_min = p->refill_threshold;
   C.tail_max = p->tail_lanes == 0 ? 8 : (p->tail_lanes < 0 ? 0 : p->tail_lanes);
   C.fused = fused ? 1 : 0;
+  C.no_unfold = replay ? 1 : 0;
   C.f64_rep = f64;
   C.take_chunk = G > 1 ? 1024u : 256u;   // at most: a warp of a batch stays on one geometry longer
   C.cell_flux_axis = p->cell_flux_axis ? 1 : 0;

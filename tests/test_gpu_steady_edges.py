@@ -1,7 +1,9 @@
 """Edges of the FP32 steady run that its usual sizes do not reach.
 
 * free paths so long that the summed tallies leave 64-bit fixed point: the
-  run's sum is that of its particles.
+  run's sum is that of its particles;
+* gradients of boxes without pore or walls whose periods do not fit one pass:
+  the replay finds the forward pass's tallies.
 """
 import numpy as np
 import pytest
@@ -34,3 +36,30 @@ def test_sum_of_tallies_is_that_of_the_particles(mfp, tail):
     # most, each within 2^-53 of the sum of magnitudes
     for k, ref, mag in ((L.STAT_SUMX, X.sum(), np.abs(X).sum()), (L.STAT_SUMX2, (X * X).sum(), (X * X).sum())):
         assert abs(o.stats[0, k].item() - ref) < 1e-12 * mag
+
+
+@pytest.mark.parametrize("tail", [0, -1])
+@pytest.mark.parametrize("axis,n", [(0, 17), (1, 17), (2, 17), (1, 40)])
+def test_two_pass_gradient_of_a_film(axis, n, tail):
+    # the film's walls across `axis`, the control gradient along it: the other
+    # two axes are periodic, and forward flights alone would run through them
+    ft, fp = [W.PERIODIC] * 6, [0.0] * 6
+    for f in {0: (W.FACE_X0, W.FACE_XL), 1: (W.FACE_Y0, W.FACE_YL), 2: (W.FACE_Z0, W.FACE_ZL)}[axis]:
+        ft[f], fp[f] = W.ADIABATIC, 0.3
+    size, grad = [100e-9] * 3, [0.0] * 3
+    size[axis] = 300e-9
+    grad[(axis + 1) % 3] = -1e6
+    g = W.Geometry(L=size, face_type=ft, face_p=fp, grad_T=tuple(grad))
+    cfg = api.SteadyConfig(seed=5, precision=L.FP32_TRACE, n_scat_max=n, tally_axis=(axis + 1) % 3, per_bin=True,
+                           max_events=10 ** 7, tail_lanes=tail)
+    M, G = api.Material(W.bvk_holland()), api.Geometry(g)
+    fwd, go = api.grad(M, G, 20_011, cfg)
+    torch.cuda.synchronize()
+    assert fwd.stats[0, L.STAT_STATUS].item() == 0 and fwd.stats[0, L.STAT_N].item() == 20_011
+    # a run without gradient takes whole flights: other roundings of the
+    # positions, which a few long trajectories turn into other events
+    run = api.run_steady(M, [G], [20_011], cfg)
+    torch.cuda.synchronize()
+    k, s = L.STAT_KAPPA, L.STAT_KAPPA_SE
+    assert abs(fwd.stats[0, k].item() - run.stats[0, k].item()) < 3 * run.stats[0, s].item()
+    assert torch.isfinite(go.dkappa_dlogtau).all()
