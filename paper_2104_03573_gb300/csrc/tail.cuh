@@ -11,6 +11,7 @@
 // gradient 1017 -> 483, square-pore mesh 1379 -> 767.
 #pragma once
 
+#include "rules.h"
 #include "tracer.cuh"
 
 namespace mcbte {

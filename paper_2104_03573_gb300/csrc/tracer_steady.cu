@@ -823,7 +823,9 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
         __syncwarp();
         if (alive) {
           const DrawLean* s0 = slots + (__popc(live & ((1u << lane) - 1u)) << sh);
-          const uint32_t e_f = p.e, nslots = ahead ? 1u << sh : 0u, e_l = p.e + (ahead ? nslots : (uint32_t)fminf(kInlineRound * per_flight, 65536.0f));
+          const uint32_t e_f = p.e, nslots = ahead ? 1u << sh : 0u;
+          const uint32_t e_l =
+              round_end(p.e, ahead ? nslots : (uint32_t)fminf(kInlineRound * per_flight, 65536.0f), C.max_events);
           const bool film = um == 3u || um == 5u || um == 6u;
           if (UNF && um && !film) {
             out = trace_unfolded(p, *G, M, relax, binf, C, key.x, key.y, T, s0, e_l, um);
