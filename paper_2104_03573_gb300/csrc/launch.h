@@ -19,18 +19,6 @@ struct SetupArgs {
   uint64_t n_norm[kMaxGeoms];
 };
 
-// Shared-memory plan of the persistent FP32 tracer.
-struct SmemPlan {
-  int relax_in_smem;   // alias records ~ C/tau in shared memory
-  int binf_in_smem;    // per-bin {v, 1/v, Lambda} in shared memory
-  int qbin_in_smem;    // frequency-resolved flux privatised per block
-  int cells_in_smem;   // cell tallies privatised per block
-  int tail_slots;      // the tail's per-thread draw slots (first in the layout)
-  int grad_in_smem;    // the gradient accumulator privatised per block
-  int snap_in_smem;    // a pore-hit snapshot per thread (measure-valued d/dp; after the tail slots)
-  size_t bytes;
-};
-
 int sm_count();
 
 // FP64 tracers: one block of six warps per SM, or fewer blocks where the run
@@ -44,13 +32,6 @@ inline int f64_blocks(uint64_t total) {
   const uint64_t most = (uint64_t)sm_count();   // a warp on every SM first
   return (int)(total < most ? total : most);
 }
-
-// Shared memory a tracer block lays out: 212 of the 227 KB it may have (the
-// rest of the SM's 256 KB is L1, which tables beyond the plan are read through).
-constexpr size_t kTableBytes = 212 * 1024;
-
-SmemPlan plan_smem_f32(int n_bins, int n_geoms, int n_cells, int per_bin, size_t budget, int tail_threads = 0,
-                       int grad_acc = 0, int snap_threads = 0);
 
 cudaError_t launch_setup(const SetupArgs& a, int n_geoms, const MatView& M, int transient, double t_max_s,
                          int tally_axis, GeoRun* geos, uint64_t* offs, unsigned long long* t0, cudaStream_t s);

@@ -11,7 +11,6 @@
 // gradient 1017 -> 483, square-pore mesh 1379 -> 767.
 #pragma once
 
-#include "rules.h"
 #include "tracer.cuh"
 
 namespace mcbte {
@@ -38,11 +37,11 @@ struct __align__(16) DrawLean : Draw32 {
   // W: the film's wall axis; s: the particle's sign
   __device__ __forceinline__ void to_film(float LW, int W, float s, int ta);
 };
-static_assert(sizeof(DrawLean) == 80, "five 16-byte words");
+static_assert(sizeof(DrawLean) == kTailSlotBytes, "five 16-byte words");
 
-// Draws a warp computes ahead at once: two per lane.  A round's fixed cost
-// (votes, the counters' shuffles, the timer) is shared by that many events.
-constexpr int kTailSlots = 64;
+// Draws a warp computes ahead at once: two per lane (kTailSlots), or one where
+// shared memory has no room for them (plan_tail).  A round's fixed cost (votes,
+// the counters' shuffles, the timer) is shared by that many events.
 
 // What the loops take of the run's parameters, by value.
 struct LoneArgs {

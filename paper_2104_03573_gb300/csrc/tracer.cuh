@@ -18,6 +18,7 @@
 #pragma once
 
 #include "mcbte_device.cuh"
+#include "rules.h"
 
 namespace mcbte {
 
@@ -264,7 +265,6 @@ __device__ __forceinline__ void resample(Particle<R>& p, const MatView& M, const
 // word: the acceptance is off by at most n / 2^32), word 1 the flight, words
 // 2 and 3 the isotropic direction.  A 24-bit flight uniform is all FP32
 // resolves.
-constexpr int kOneBlockBins = 65536;
 
 // ------------------------------------------------------------------ FP32 event draws
 // What the words of one event decide whatever the particle's state (FP32

@@ -616,15 +616,15 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   long long* s_qbin = nullptr;
   long long* s_cP = nullptr;
   long long* s_cD = nullptr;
-  // the warps' emitted batches (main kernel) or the tail kernel's draw slots,
-  // 32 per warp, come first (16-byte aligned)
+  // the warps' emitted batches (main kernel) or the tail kernel's draw slots
+  // come first (16-byte aligned)
   using RefillT = Refill<float, EXT, false>;
   RefillT& refill = reinterpret_cast<RefillT*>(sp)[threadIdx.x >> 5];
   if constexpr (!TK) sp += (TPB / 32) * sizeof(RefillT);
   DrawLean* slots = nullptr;
-  if (TK && S.tail_slots) {
-    slots = reinterpret_cast<DrawLean*>(sp) + (size_t)(threadIdx.x >> 5) * kTailSlots;
-    sp += (size_t)(TPB / 32) * kTailSlots * sizeof(DrawLean);
+  if (TK) {
+    slots = reinterpret_cast<DrawLean*>(sp) + (size_t)(threadIdx.x >> 5) * S.tail_slots;
+    sp += (size_t)(TPB / 32) * S.tail_slots * sizeof(DrawLean);
   }
   // then the pore-hit snapshots (16-byte aligned), four int4 per thread
   int4* snaps = nullptr;
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   const uint2 key = run_key(C);
   const int refill_min = (C.refill_min > 1 && !TK) ? C.refill_min : 1;
   // the tail: parking (main kernel) or the draws ahead (tail kernel)
-  const int tail_max = (TK ? (slots != nullptr && n <= kOneBlockBins) : (MODE == 1 && A.park_cap > 0)) ? C.tail_max : 0;
+  const int tail_max = (TK ? n <= kOneBlockBins : (MODE == 1 && A.park_cap > 0)) ? C.tail_max : 0;
   const uint64_t n_parked = TK ? min(*(volatile unsigned long long*)A.park_n, (unsigned long long)A.park_cap) : 0;
   bool pool_dry = false;   // the same in every lane: nothing left to hand out
   if constexpr (!TK) refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
@@ -769,8 +769,8 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
         }
         continue;   // lanes the buffer could not take trace on with the next votes (park_cap reached)
       } else {
-        // log2 of the slots per particle: nlive << sh <= kTailSlots
-        const int sh = (kTailSlots == 64 ? 6 : 5) - (32 - __clz(nlive - 1));
+        // log2 of the slots per particle: nlive << sh <= S.tail_slots
+        const int sh = (31 - __clz(S.tail_slots)) - (32 - __clz(nlive - 1));
         const unsigned um = (UNF && alive) ? unfold_mask<GradT>(*G, C) : 0u;
         // draws ahead, or (most of the live particles in thick films) inline
         bool ahead = true;
@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
         }
 #pragma unroll
         for (int h = 0; h < kTailSlots / 32; ++h) {
-          if (!ahead) break;
+          if (!ahead || 32 * h >= S.tail_slots) break;
           const unsigned i = lane + 32u * h;
           const int r = (int)(i >> sh);   // the live particle slot i belongs to
           // its lane: a lone particle's is the only one, else the r-th live lane
@@ -1179,8 +1179,9 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
   // the gradient kernel keeps no cell tallies, and the per-bin flux only in
   // a fused pass
   constexpr size_t kBatch = MODE == 2 ? 0 : (TPB / 32) * sizeof(Refill<float, EXT, false>);
-  SmemPlan S = plan_smem_f32(M.n, C.n_geoms, GRAD ? 0 : C.n_cells, (GRAD && !C.fused) ? 0 : C.per_bin,
-                                   kTableBytes - kBatch, MODE == 2 ? TPB : 0, GRAD ? 1 : 0, (GRAD && C.mvd) ? TPB : 0);
+  const int nc = GRAD ? 0 : C.n_cells, pb = (GRAD && !C.fused) ? 0 : C.per_bin, snaps = (GRAD && C.mvd) ? TPB : 0;
+  SmemPlan S = MODE == 2 ? plan_tail(M.n, C.n_geoms, nc, pb, GRAD ? 1 : 0, snaps)
+                         : plan_tables(M.n, C.n_geoms, nc, pb, 212 * 1024 - kBatch, GRAD ? 1 : 0, snaps);
   S.bytes += kBatch;
   auto kern = k_steady_f32<CELLS, GRAD, TPB, EXT, MODE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.bytes);
@@ -1204,9 +1205,6 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
 
 // Part 0: the main kernel alone.  Part 1: the main kernel that parks its
 // tail, then the tail kernel over the parked particles (256-thread blocks).
-#if MCBTE_F32_PART == 1
-constexpr int kTailThreads = 256;
-#endif
 
 template <int CELLS, bool GRAD, int TPB, bool EXT>
 cudaError_t launch_f32_tpb(const GeoRun* geos, const uint64_t* offs, const MatView& M, const RunCfg& C,
@@ -1253,50 +1251,6 @@ cudaError_t launch_f32_variants(bool grad, bool cells, const GeoRun* geos, const
 }  // namespace
 
 #if MCBTE_F64
-SmemPlan plan_smem_f32(int n_bins, int n_geoms, int n_cells, int per_bin, size_t budget, int tail_threads,
-                       int grad_acc, int snap_threads) {
-  // By use per event: the relaxation alias records and the per-bin
-  // constants (every relaxation), the cell tallies (every flight), the
-  // per-bin flux (every relaxation period), the gradient accumulator (every
-  // period of a gradient pass); each is placed while room remains, then the
-  // tail's draw slots (kTailSlots DrawLean per warp), then the pore-hit snapshots
-  // of the measure-valued d/dp (64 bytes per thread).
-  SmemPlan S{0, 0, 0, 0, 0, 0, 0, 0};
-  size_t used = 0;
-  if (used + (size_t)n_bins * 16 <= budget) {
-    S.relax_in_smem = 1;
-    used += (size_t)n_bins * 16;
-  }
-  if (used + (size_t)n_bins * 16 <= budget) {
-    S.binf_in_smem = 1;
-    used += (size_t)n_bins * 16;
-  }
-  const size_t cells = (size_t)(n_cells * 4 + (n_cells + 1) * 4) * sizeof(long long);
-  if (n_cells > 0 && n_geoms == 1 && used + cells <= budget) {
-    S.cells_in_smem = 1;
-    used += cells;
-  }
-  if (per_bin && n_geoms == 1 && used + (size_t)n_bins * 8 <= budget) {
-    S.qbin_in_smem = 1;
-    used += (size_t)n_bins * 8;
-  }
-  if (grad_acc && used + (size_t)n_bins * 8 <= budget) {
-    S.grad_in_smem = 1;
-    used += (size_t)n_bins * 8;
-  }
-  const size_t slots = (size_t)(tail_threads / 32) * kTailSlots * sizeof(DrawLean);
-  if (tail_threads > 0 && n_bins <= kOneBlockBins && used + slots <= budget) {
-    S.tail_slots = 1;
-    used += slots;
-  }
-  if (snap_threads > 0 && used + (size_t)snap_threads * 4 * sizeof(int4) <= budget) {
-    S.snap_in_smem = 1;
-    used += (size_t)snap_threads * 4 * sizeof(int4);
-  }
-  S.bytes = used;
-  return S;
-}
-
 // SM count of the current device, cached per device ordinal (grids are sized
 // for the device the launch goes to).
 int sm_count() {

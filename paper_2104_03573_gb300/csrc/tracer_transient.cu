@@ -693,7 +693,7 @@ cudaError_t launch_transient_tav(const GeoRun* geos, const MatView& M, const Run
                                  cudaStream_t s) {
   const size_t tm_bytes = (((size_t)C.n_times * sizeof(float) + 15) & ~(size_t)15) +
                           (TAVG ? 0 : (TPB / 32) * sizeof(FlightSlots));
-  SmemPlan S = plan_smem_f32(M.n, 1, 0, 0, 200 * 1024 - tm_bytes);
+  SmemPlan S = plan_tables(M.n, 1, 0, 0, 200 * 1024 - tm_bytes);
   S.bytes += tm_bytes;
   auto kern = k_transient_f32<TPB, EXT, TAVG>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.bytes);

@@ -3,7 +3,9 @@
 * free paths so long that the summed tallies leave 64-bit fixed point: the
   run's sum is that of its particles;
 * gradients of boxes without pore or walls whose periods do not fit one pass:
-  the replay finds the forward pass's tallies.
+  the replay finds the forward pass's tallies;
+* bin counts whose tables leave the tail 32 draw slots per warp, or no room for
+  a table: the same bits as without the tail.
 """
 import numpy as np
 import pytest
@@ -63,3 +65,42 @@ def test_two_pass_gradient_of_a_film(axis, n, tail):
     k, s = L.STAT_KAPPA, L.STAT_KAPPA_SE
     assert abs(fwd.stats[0, k].item() - run.stats[0, k].item()) < 3 * run.stats[0, s].item()
     assert torch.isfinite(go.dkappa_dlogtau).all()
+
+
+# with the per-bin flux: 4110 bins leave a gradient 32 slots, 5100 a forward
+# run; at 6300 and 12 600 the flux, and the per-bin constants, are in global memory
+@pytest.mark.parametrize("bins", [4110, 5100, 6300, 12_600])
+@pytest.mark.parametrize("kind", ["film", "pore", "walls", "batch"])
+def test_tails_at_bin_counts_between(kind, bins):
+    M = api.Material(W.bvk_holland(n_per_branch=bins // 3))
+    assert M.n_bins == bins
+    gs = {"film": [W.film(100e-9, p=0.4)], "pore": [W.pore_lattice(100e-9, 0.25, 200e-9, p_pore=0.4)],
+          "walls": [W.nanomesh(p_pore=0.4)], "batch": [W.film(30e-9), W.film(2000e-9), W.film(200e-9)]}[kind]
+    outs = []
+    for tail in (-1, 8):
+        cfg = api.SteadyConfig(seed=45, precision=L.FP32_TRACE, tally_axis=1, n_scat_max=10, per_bin=True,
+                               max_events=10 ** 6, tail_lanes=tail)
+        o = api.run_steady(M, [api.Geometry(g) for g in gs], [5003] * len(gs), cfg, per_particle=True)
+        torch.cuda.synchronize()
+        outs.append([getattr(o, k).cpu().numpy() for k in ("events_pp", "X_pp", "q_bin")])
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("bins", [4110, 5100, 6300, 12_600])
+@pytest.mark.parametrize("p", [0.0, 0.4])
+def test_gradient_tails_at_bin_counts_between(p, bins):
+    M = api.Material(W.bvk_holland(n_per_branch=bins // 3))
+    G = api.Geometry(W.pore_lattice(100e-9, 0.25, 200e-9, p_pore=p))
+    outs = []
+    for tail in (-1, 8):
+        cfg = api.SteadyConfig(seed=46, precision=L.FP32_TRACE, tally_axis=1, n_scat_max=10, per_bin=True,
+                               max_events=10 ** 6, tail_lanes=tail)
+        fwd, go = api.grad(M, G, 5003, cfg)
+        torch.cuda.synchronize()
+        assert fwd.stats[0, L.STAT_N].item() == 5003
+        outs.append([t.cpu().numpy() for t in (fwd.q_bin, go.dkappa_dlogtau, go.dkappa_dp)])
+    # the same particles: whole-number sums equal, FP64 sums over particles in another order
+    assert np.array_equal(outs[0][0], outs[1][0])
+    for a, b in zip(outs[0][1:], outs[1][1:]):
+        assert np.max(np.abs(a - b)) < 1e-9 * np.max(np.abs(a))
