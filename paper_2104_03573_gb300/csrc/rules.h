@@ -34,7 +34,8 @@ struct SmemPlan {
   int cells_in_smem;   // cell tallies privatised per block
   int tail_slots;      // the tail's draw slots per warp, 0 without (first in the layout)
   int grad_in_smem;    // the gradient accumulator privatised per block
-  int snap_in_smem;    // a pore-hit snapshot per thread (measure-valued d/dp; after the tail slots)
+  int snap_in_smem;    // a pore-hit snapshot per thread (measure-valued d/dp; after the warps' records)
+  int batch_slots;     // the main kernel's emitted batch: slots per warp, 0 without (first in the layout)
   size_t bytes;
 };
 
@@ -46,7 +47,7 @@ struct SmemPlan {
 // remains in `budget`.
 inline SmemPlan plan_tables(int n_bins, int n_geoms, int n_cells, int per_bin, size_t budget, int grad_acc = 0,
                             int snap_threads = 0) {
-  SmemPlan S{0, 0, 0, 0, 0, 0, 0, 0};
+  SmemPlan S{0, 0, 0, 0, 0, 0, 0, 0, 0};
   auto place = [&](bool wanted, size_t bytes) {
     const bool in = wanted && S.bytes + bytes <= budget;
     if (in) S.bytes += bytes;
@@ -85,6 +86,29 @@ inline SmemPlan plan_tail(int n_bins, int n_geoms, int n_cells, int per_bin, int
   if (n_bins > kOneBlockBins) return S;
   S.tail_slots = S.bytes + kTailSlots * slot <= kPlanBytes ? kTailSlots : kTailSlots / 2;
   S.bytes += (size_t)S.tail_slots * slot;
+  return S;
+}
+
+// The main kernel's emitted batches (Refill, EmitBatch): 32 slots per warp
+// where they fit beside the tables, else 16.  A table or tally in global memory
+// costs far more (silicon-like slab, 2e6 particles, 50 cells: 5700 bins
+// 139 ms with 32 slots and the cells outside, 5.5 with 16; 4650 bins 13.4 ms
+// with the per-bin flux outside, 5.8).  Blocks of 1024 threads take none: their
+// 64 registers spill with them, into the L1 whose room they take (the same
+// slab, 1e7 particles, 3000 / 4200 / 7800 bins: 18.7 / 24.9 / 27.3 ms with,
+// 16.9 / 17.3 / 17.9 without).
+constexpr int kUnbatchedThreads = 1024;   // and more
+constexpr int kBatchSlots = 32;
+constexpr size_t kRefillBytes = 48, kBatchBytes = 1296, kBatchBytesExt = 1424;   // a record holds 32 slots
+
+inline SmemPlan plan_main(int threads, bool ext, int n_bins, int n_geoms, int n_cells, int per_bin, int grad_acc,
+                          int snap_threads) {
+  SmemPlan S = plan_tables(n_bins, n_geoms, n_cells, per_bin, kTableBytes, grad_acc, snap_threads);
+  if (threads >= kUnbatchedThreads) return S;
+  const size_t warps = (size_t)(threads / 32), rec = ext ? kBatchBytesExt : kBatchBytes;
+  auto bytes = [&](int slots) { return warps * kRefillBytes + (warps * (size_t)slots / kBatchSlots) * rec; };
+  S.batch_slots = S.bytes + bytes(kBatchSlots) <= kPlanBytes ? kBatchSlots : kBatchSlots / 2;
+  S.bytes += bytes(S.batch_slots);
   return S;
 }
 

@@ -1029,10 +1029,10 @@ struct WarpRun {
     if (nb + chunk >= total) dry = true;
     return k;
   }
-  // The next consecutive indices, 32 at most: their first one, and how many
+  // The next consecutive indices, `most` at most: their first one, and how many
   // (0: the run has no more).  Called by the whole warp.
-  __device__ __forceinline__ uint64_t batch(unsigned lane, unsigned long long* work, uint64_t total, uint64_t deadline,
-                                            int* flags, int* count) {
+  __device__ __forceinline__ uint64_t batch(int most, unsigned lane, unsigned long long* work, uint64_t total,
+                                            uint64_t deadline, int* flags, int* count) {
     if (cb >= ce && !dry) {
       unsigned long long nb = 0;
       if (lane == 0) {
@@ -1046,7 +1046,7 @@ struct WarpRun {
     }
     const uint64_t first = cb;
     const uint64_t left = cb < ce ? ce - cb : 0;
-    *count = left < 32 ? (int)left : 32;
+    *count = left < (unsigned)most ? (int)left : most;
     cb += (unsigned)*count;
     return first;
   }
@@ -1054,13 +1054,15 @@ struct WarpRun {
 };
 
 // Particles a warp has emitted and not yet handed to a lane, one batch of 32
-// consecutive indices (shared memory, a word per lane and field).  Emission
+// consecutive indices (shared memory, a word per slot and field).  Emission
 // takes three to four Philox blocks and two table reads; emitting for the few
 // lanes that wait left the other lanes idle meanwhile, and waiting for more of
 // them cost lanes too.  A batch is emitted by all 32 lanes at once and a lane
-// refills by a few shared-memory reads.
+// refills by a few shared-memory reads.  Where 32 slots per warp would push a
+// table out of shared memory two warps share a record, 16 slots each
+// (plan_main): the fields keep their fixed distances, which cost no registers.
 template <typename R, bool EXT, bool TR>
-struct EmitBatch {
+struct __align__(16) EmitBatch {
   R x[3][32], u[3][32], d_rel[32];
   R d2[EXT ? 32 : 1];
   R t[TR ? 32 : 1];
@@ -1100,34 +1102,39 @@ struct EmitBatch {
   }
 };
 
-// One particle emitted into slot `lane` of a warp's batch.
-template <typename R, bool EXT, bool TR>
-__device__ __forceinline__ void emit_slot(EmitBatch<R, EXT, TR>* b, unsigned lane, const GeoRun* geos,
-                                          const uint64_t* offs, int n_geoms, uint64_t idx, const MatView& M,
-                                          const float4* binf, uint2 key, R t_max_ps) {
-  int lo = 0, hi = n_geoms;
+// Geometry of particle idx of a run: offs[g] <= idx < offs[g + 1].
+__device__ __forceinline__ int find_geom(const uint64_t* offs, int G, uint64_t idx) {
+  int lo = 0, hi = G;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (offs[mid] <= idx) lo = mid; else hi = mid;
   }
-  const GeoRun& G = geos[lo];
-  Particle<R> p;
-  p.pid = (uint32_t)(idx - (n_geoms > 1 ? offs[lo] : 0) + G.pid0);
-  p.g = lo;
-  emit<R, EXT>(p, G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, TR, t_max_ps);
-  b->store(lane, p);
+  return lo;
 }
 
-// A warp's refill: its run of particle indices, and the batch it emitted last.
-// All of it in shared memory, read once per refill: as registers the
-// warp-uniform state took a dozen of every thread's.  hand_out() gives the
-// lanes in `want` the next particles of the batch and emits new ones as they
-// run out; emit_one(index) emits into the lane's slot, and take(slot, index)
-// is called in each lane that gets one.  Returns whether the run has nothing
-// left for the warp (or its time budget is over).
+// One particle emitted into slot `i` of a batch.
 template <typename R, bool EXT, bool TR>
+__device__ __forceinline__ void emit_slot(EmitBatch<R, EXT, TR>* b, unsigned i, const GeoRun* geos,
+                                          const uint64_t* offs, int n_geoms, uint64_t idx, const MatView& M,
+                                          const float4* binf, uint2 key, R t_max_ps) {
+  const int g = find_geom(offs, n_geoms, idx);
+  const GeoRun& G = geos[g];
+  Particle<R> p;
+  p.pid = (uint32_t)(idx - (n_geoms > 1 ? offs[g] : 0) + G.pid0);
+  p.g = g;
+  emit<R, EXT>(p, G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, TR, t_max_ps);
+  b->store(i, p);
+}
+
+// A warp's refill: its run of particle indices, and how far the batch it
+// emitted last is handed out.  All of it in shared memory, read once per
+// refill: as registers the warp-uniform state took a dozen of every thread's.
+// hand_out() gives the lanes in `want` the next particles of the batch and
+// emits new ones, `slots` at most, as they run out; emit_one(index) emits into
+// the lane's slot, and take(slot, index) is called in each lane that gets one.
+// Returns whether the run has nothing left for the warp (or its time budget is
+// over).
 struct Refill {
-  EmitBatch<R, EXT, TR> b;
   WarpRun run;
   uint64_t first;   // particle index of the batch's first
   int next, n;
@@ -1145,14 +1152,14 @@ struct Refill {
   }
 
   template <class Emit, class Take>
-  __device__ __forceinline__ bool hand_out(unsigned want, unsigned lane, unsigned long long* work, uint64_t total,
-                                           uint64_t deadline, int* flags, Emit emit_one, Take take) {
+  __device__ __forceinline__ bool hand_out(int slots, unsigned want, unsigned lane, unsigned long long* work,
+                                           uint64_t total, uint64_t deadline, int* flags, Emit emit_one, Take take) {
     constexpr unsigned kAll = 0xffffffffu;
     int at = next, cnt_b = n;
     for (;;) {
       if (at == cnt_b) {
         WarpRun r = run;
-        const uint64_t f = r.batch(lane, work, total, deadline, flags, &cnt_b);
+        const uint64_t f = r.batch(slots, lane, work, total, deadline, flags, &cnt_b);
         const int stop = *(volatile int*)flags & 1;
         if (cnt_b == 0 || __any_sync(kAll, stop)) return true;
         at = 0;
@@ -1181,6 +1188,10 @@ struct Refill {
     return done;
   }
 };
+
+static_assert(sizeof(Refill) == kRefillBytes && sizeof(EmitBatch<float, false, false>) == kBatchBytes &&
+                  sizeof(EmitBatch<float, true, false>) == kBatchBytesExt,
+              "the plan's sizes");
 
 // Philox key of the run: the host seed, or the device-resident one.
 __device__ __forceinline__ uint2 run_key(const RunCfg& C) {

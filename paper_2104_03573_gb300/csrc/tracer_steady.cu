@@ -27,15 +27,6 @@ namespace mcbte {
 
 namespace {
 
-__device__ __forceinline__ int find_geom(const uint64_t* offs, int G, uint64_t idx) {
-  int lo = 0, hi = G;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (offs[mid] <= idx) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 // N_scat_max curve: a trajectory that ended (absorbed, truncated) after m <
 // n_scat_max relaxations has the same final tally X in every run with
 // N_scat_max > m; it enters the difference array at m + 1.
@@ -241,7 +232,8 @@ template <bool CELLS, bool GRAD>
 __global__ void __launch_bounds__(kF64Threads, 1) k_steady_fp64(const GeoRun* __restrict__ geos,
                                                                 const uint64_t* __restrict__ offs, MatView M, RunCfg C,
                                                                 Acc A) {
-  __shared__ Refill<double, true, false> s_refill[kF64Threads / 32];
+  __shared__ Refill s_refill[kF64Threads / 32];
+  __shared__ EmitBatch<double, true, false> s_batch[kF64Threads / 32];
   __shared__ BlockAcct<double> s_acct;
   if (threadIdx.x == 0) s_acct.reset();
   __syncthreads();
@@ -249,7 +241,8 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_steady_fp64(const GeoRun* __
   const unsigned lane = threadIdx.x & 31u;
   const uint64_t deadline = *C.t0 + C.budget_ns;
   const uint2 key = run_key(C);
-  Refill<double, true, false>& refill = s_refill[threadIdx.x >> 5];
+  Refill& refill = s_refill[threadIdx.x >> 5];
+  EmitBatch<double, true, false>& batch = s_batch[threadIdx.x >> 5];
   refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
   Particle<double> p;
   using GradT = typename GradPick<GRAD, GradList>::type;
@@ -273,12 +266,12 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_steady_fp64(const GeoRun* __
     const unsigned need = __ballot_sync(kAll, !alive);
     if (need && !pool_dry) {
       pool_dry = refill.hand_out(
-          need, lane, A.work, C.total, deadline, A.flags,
+          32, need, lane, A.work, C.total, deadline, A.flags,
           [&](uint64_t k) {
-            emit_slot<double, true, false>(&refill.b, lane, geos, offs, C.n_geoms, k, M, nullptr, key, 0.0);
+            emit_slot<double, true, false>(&batch, lane, geos, offs, C.n_geoms, k, M, nullptr, key, 0.0);
           },
           [&](unsigned slot, uint64_t) {
-            refill.b.load(slot, p, M, nullptr);
+            batch.load(slot, p, M, nullptr);
             if (p.g != acct.g) {
               acct.flush(A);
               acct.reset(p.g);
@@ -570,7 +563,9 @@ __device__ __forceinline__ int trace_unfolded(Particle<float>& p, const GeoRun& 
 // lanes alone took 150 warp instructions a particle; what made room for the
 // batch at 80 registers a thread is that nothing a particle needs once (the
 // lane's book-keeping, the warp's run) stays in registers.  1e7-particle
-// silicon-like slab: 17.98 -> 15.32 ms.
+// silicon-like slab: 17.98 -> 15.32 ms.  Blocks of 1024 threads have 64
+// registers, which the batch made the event loop spill, and the batches' room
+// is the L1's: their lanes emit for themselves (kUnbatchedThreads).
 // TPB is the block size the kernel is compiled for (register budget).
 // GRAD: the gradient pass.  Fused (C.fused): the forward run's tallies,
 // counters and per-particle outputs and the gradient in one pass, each
@@ -618,9 +613,14 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   long long* s_cD = nullptr;
   // the warps' emitted batches (main kernel) or the tail kernel's draw slots
   // come first (16-byte aligned)
-  using RefillT = Refill<float, EXT, false>;
-  RefillT& refill = reinterpret_cast<RefillT*>(sp)[threadIdx.x >> 5];
-  if constexpr (!TK) sp += (TPB / 32) * sizeof(RefillT);
+  constexpr bool kBatched = !TK && TPB < kUnbatchedThreads;
+  using BatchT = EmitBatch<float, EXT, false>;
+  Refill& refill = reinterpret_cast<Refill*>(sp)[threadIdx.x >> 5];
+  const unsigned slot_at = (threadIdx.x >> 5) * (unsigned)S.batch_slots;   // the warp's first, over all records
+  BatchT& batch = reinterpret_cast<BatchT*>(sp + (TPB / 32) * sizeof(Refill))[slot_at / kBatchSlots];
+  const unsigned slot0 = slot_at % kBatchSlots;
+  if constexpr (kBatched)
+    sp += (TPB / 32) * sizeof(Refill) + ((TPB / 32) * (unsigned)S.batch_slots / kBatchSlots) * sizeof(BatchT);
   DrawLean* slots = nullptr;
   if (TK) {
     slots = reinterpret_cast<DrawLean*>(sp) + (size_t)(threadIdx.x >> 5) * S.tail_slots;
@@ -723,7 +723,9 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
   const int tail_max = (TK ? n <= kOneBlockBins : (MODE == 1 && A.park_cap > 0)) ? C.tail_max : 0;
   const uint64_t n_parked = TK ? min(*(volatile unsigned long long*)A.park_n, (unsigned long long)A.park_cap) : 0;
   bool pool_dry = false;   // the same in every lane: nothing left to hand out
-  if constexpr (!TK) refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
+  WarpRun run;   // without a batch: the warp's particle indices not yet handed out
+  if constexpr (kBatched) refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
+  else if constexpr (!TK) run.start(C.take_chunk, C.total, deadline, A.flags);
   // a particle's index in the run
   auto index_of = [&](const Particle<float>& q) { return offs[q.g] + (q.pid - (uint32_t)geos[q.g].pid0); };
   // the tallies of the lane's geometry
@@ -870,14 +872,33 @@ __global__ void __launch_bounds__(TPB, 1) k_steady_f32(const GeoRun* __restrict_
             }
             alive = true;
           }
+        } else if constexpr (!kBatched) {
+          const uint64_t k = run.take(need, lane, A.work, C.total, deadline, A.flags);
+          if (run.empty()) pool_dry = true;
+          if (!alive && !drained) {
+            if (k >= C.total || (*(volatile int*)A.flags & 1)) {
+              drained = true;
+              continue;
+            }
+            const int g = find_geom(offs, C.n_geoms, k);
+            bind(g);
+            p.pid = (uint32_t)(k - offs[g] + G->pid0);
+            p.g = g;
+            emit<float, EXT>(p, *G, M, M.rec_emit, M.rec_init, binf, key.x, key.y, false, 0.0f);
+            if constexpr (GRAD) {
+              gr.init(p.bin);
+              if (!C.fused) gr.Xf = A.X_pp[k];
+            }
+            alive = true;
+          }
         } else {
           pool_dry = refill.hand_out(
-              need, lane, A.work, C.total, deadline, A.flags,
+              S.batch_slots, need, lane, A.work, C.total, deadline, A.flags,
               [&](uint64_t k) {
-                emit_slot<float, EXT, false>(&refill.b, lane, geos, offs, C.n_geoms, k, M, binf, key, 0.0f);
+                emit_slot<float, EXT, false>(&batch, slot0 + lane, geos, offs, C.n_geoms, k, M, binf, key, 0.0f);
               },
               [&](unsigned slot, uint64_t k) {
-                refill.b.load(slot, p, M, binf);
+                batch.load(slot0 + slot, p, M, binf);
                 bind(p.g);
                 if constexpr (GRAD) {
                   gr.init(p.bin);
@@ -1178,11 +1199,9 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
                               const Acc& A, int bps, cudaStream_t s) {
   // the gradient kernel keeps no cell tallies, and the per-bin flux only in
   // a fused pass
-  constexpr size_t kBatch = MODE == 2 ? 0 : (TPB / 32) * sizeof(Refill<float, EXT, false>);
   const int nc = GRAD ? 0 : C.n_cells, pb = (GRAD && !C.fused) ? 0 : C.per_bin, snaps = (GRAD && C.mvd) ? TPB : 0;
-  SmemPlan S = MODE == 2 ? plan_tail(M.n, C.n_geoms, nc, pb, GRAD ? 1 : 0, snaps)
-                         : plan_tables(M.n, C.n_geoms, nc, pb, 212 * 1024 - kBatch, GRAD ? 1 : 0, snaps);
-  S.bytes += kBatch;
+  const SmemPlan S = MODE == 2 ? plan_tail(M.n, C.n_geoms, nc, pb, GRAD ? 1 : 0, snaps)
+                               : plan_main(TPB, EXT, M.n, C.n_geoms, nc, pb, GRAD ? 1 : 0, snaps);
   auto kern = k_steady_f32<CELLS, GRAD, TPB, EXT, MODE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.bytes);
   if (e != cudaSuccess) return e;

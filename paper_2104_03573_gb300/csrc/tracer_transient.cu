@@ -76,13 +76,15 @@ struct WarpAcct {
 // is done refills.
 __global__ void __launch_bounds__(kF64Threads, 1) k_transient_fp64(const GeoRun* __restrict__ geos, MatView M, RunCfg C,
                                                                    Acc A) {
-  __shared__ Refill<double, true, true> s_refill[kF64Threads / 32];
+  __shared__ Refill s_refill[kF64Threads / 32];
+  __shared__ EmitBatch<double, true, true> s_batch[kF64Threads / 32];
   constexpr unsigned kAll = 0xffffffffu;
   const unsigned lane = threadIdx.x & 31u;
   const GeoRun& G = geos[0];
   const uint64_t deadline = *C.t0 + C.budget_ns;
   const uint2 key = run_key(C);
-  Refill<double, true, true>& refill = s_refill[threadIdx.x >> 5];
+  Refill& refill = s_refill[threadIdx.x >> 5];
+  EmitBatch<double, true, true>& batch = s_batch[threadIdx.x >> 5];
   refill.start(lane, C.take_chunk, C.total, deadline, A.flags);
   Particle<double> p;
   p.e = 0u;
@@ -93,12 +95,12 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_transient_fp64(const GeoRun*
     const unsigned need = __ballot_sync(kAll, !alive);
     if (need && !pool_dry) {
       pool_dry = refill.hand_out(
-          need, lane, A.work, C.total, deadline, A.flags,
+          32, need, lane, A.work, C.total, deadline, A.flags,
           [&](uint64_t k) {
-            emit_slot<double, true, true>(&refill.b, lane, geos, nullptr, 1, k, M, nullptr, key, C.t_max_ps);
+            emit_slot<double, true, true>(&batch, lane, geos, nullptr, 1, k, M, nullptr, key, C.t_max_ps);
           },
           [&](unsigned slot, uint64_t) {
-            refill.b.load(slot, p, M, nullptr);
+            batch.load(slot, p, M, nullptr);
             transient_start(p, C);
             alive = true;
           });

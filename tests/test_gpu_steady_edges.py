@@ -5,7 +5,9 @@
 * gradients of boxes without pore or walls whose periods do not fit one pass:
   the replay finds the forward pass's tallies;
 * bin counts whose tables leave the tail 32 draw slots per warp, or no room for
-  a table: the same bits as without the tail.
+  a table: the same bits as without the tail;
+* bin counts whose tables leave a warp's batch 16 slots: the same bits in every
+  launch shape.
 """
 import numpy as np
 import pytest
@@ -104,3 +106,25 @@ def test_gradient_tails_at_bin_counts_between(p, bins):
     assert np.array_equal(outs[0][0], outs[1][0])
     for a, b in zip(outs[0][1:], outs[1][1:]):
         assert np.max(np.abs(a - b)) < 1e-9 * np.max(np.abs(a))
+
+
+# with per-bin flux 4800 bins leave blocks of 768 threads 32 slots, 5010 16;
+# without it 5850 and 6390
+@pytest.mark.parametrize("bins,per_bin", [(4800, True), (5010, True), (5850, False), (6390, False)])
+@pytest.mark.parametrize("walls", [False, True])
+@pytest.mark.parametrize("n", [1, 33, 20_011])
+def test_batches_at_bin_counts_between(n, walls, bins, per_bin):
+    M = api.Material(W.bvk_holland(n_per_branch=bins // 3))
+    G = api.Geometry(W.nanomesh(p_pore=0.4) if walls else W.slab_z(1e-6, 300.5, 299.5, lateral=1e-6))
+    base = None
+    for threads in (256, 512, 768, 1024):
+        cfg = api.SteadyConfig(seed=47, precision=L.FP32_TRACE, tally_axis=1 if walls else 2, n_cells=33, cell_axis=2,
+                               n_scat_max=10 if walls else 0, per_bin=per_bin, max_events=10 ** 6,
+                               threads_per_block=threads)
+        o = api.run_steady(M, [G], [n], cfg, per_particle=True)
+        torch.cuda.synchronize()
+        assert o.stats[0, L.STAT_N].item() == n
+        cur = [getattr(o, k).cpu().numpy() for k in ("events_pp", "X_pp", "T", "q") + (("q_bin",) if per_bin else ())]
+        base = base or cur
+        for a, b in zip(base, cur):
+            assert np.array_equal(a, b), threads

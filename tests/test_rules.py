@@ -2,7 +2,8 @@
 
 * a round of the tail's events always goes on, up to the last event number;
 * the tail kernel has draw slots at every bin count, and every table that has
-  room in 200 KB without them.
+  room in 200 KB without them;
+* so have the main kernel's warps their batches, in blocks below 1024 threads.
 """
 import os
 import subprocess
@@ -24,7 +25,7 @@ int main() {
   auto take = [&](int k) { for (int i = 0; i < k; ++i) if (scanf("%u", &a[i]) != 1) exit(1); };
   auto show = [](const SmemPlan& S) {
     printf("%d %d %d %d %d %d %d %zu\n", S.relax_in_smem, S.binf_in_smem, S.cells_in_smem, S.qbin_in_smem,
-           S.grad_in_smem, S.snap_in_smem, S.tail_slots, S.bytes);
+           S.grad_in_smem, S.snap_in_smem, S.tail_slots + S.batch_slots, S.bytes);
   };
   while (scanf("%31s", rule) == 1) {
     if (!strcmp(rule, "round_end")) {
@@ -33,6 +34,9 @@ int main() {
     } else if (!strcmp(rule, "plan_tail")) {
       take(6);
       show(plan_tail(a[0], a[1], a[2], a[3], a[4], a[5]));
+    } else if (!strcmp(rule, "plan_main")) {
+      take(8);
+      show(plan_main(a[0], a[1] != 0, a[2], a[3], a[4], a[5], a[6], a[7]));
     }
   }
   return 0;
@@ -99,3 +103,23 @@ def test_tail_plan_has_slots_and_tables_at_every_bin_count(rules, G, nc, pb, gra
             continue
         assert slots == (64 if used + 64 * 8 * 80 <= 226 * KB else 32), n
         assert g[7] == used + slots * 8 * 80 <= 226 * KB
+
+
+@pytest.mark.parametrize("G,nc,pb,grad,snap", ASKS)
+@pytest.mark.parametrize("threads", [256, 512, 768, 1024])
+@pytest.mark.parametrize("ext", [0, 1])
+def test_main_plan_has_batches_and_tables_at_every_bin_count(rules, ext, threads, G, nc, pb, grad, snap):
+    snap = threads if snap else 0
+    got = rules("plan_main", [(threads, ext, n, G, nc, pb, grad, snap) for n in BINS])
+    warps, rec = threads // 32, 1424 if ext else 1296
+    for n, g in zip(BINS, got):
+        res, used = _tables(n, G, nc, pb, grad, snap)
+        assert g[:6] == res, n
+        slots = g[6]
+        if threads == 1024:
+            assert slots == 0 and g[7] == used
+            continue
+        assert slots == (32 if used + warps * (48 + rec) <= 226 * KB else 16), n
+        # two warps share a record of 32 slots where each has 16; the tables behind them are 16-byte aligned
+        front = warps * 48 + warps * slots // 32 * rec
+        assert front % 16 == 0 and g[7] == used + front <= 226 * KB
