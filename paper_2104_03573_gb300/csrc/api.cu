@@ -687,6 +687,9 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
     a.pid0[g] = p->pid_begin ? p->pid_begin[g] : 0;
     a.n_norm[g] = p->n_total ? p->n_total[g] : p->n_particles[g];
   }
+  // forward pass of a two-pass gradient: flights stop at periodic faces, as the
+  // replay's do (the rounding of a flight's tally depends on its cuts)
+  a.cut_flights = replay ? 1 : 0;
   RUN_TRY(launch_setup(a, G, m->view, 0, 0.0, p->tally_axis, w.geos, w.offs, w.t0, s));
   RunCfg C{};
   C.k0 = (uint32_t)p->seed;
@@ -705,7 +708,6 @@ mcbte_status steady_impl(const mcbte_material* m, const mcbte_geometry* const* g
   C.refill_min = p->refill_threshold;
   C.tail_max = p->tail_lanes == 0 ? 8 : (p->tail_lanes < 0 ? 0 : p->tail_lanes);
   C.fused = fused ? 1 : 0;
-  C.no_unfold = replay ? 1 : 0;
   C.f64_rep = f64;
   C.take_chunk = G > 1 ? 1024u : 256u;   // at most: a warp of a batch stays on one geometry longer
   C.cell_flux_axis = p->cell_flux_axis ? 1 : 0;

@@ -17,6 +17,7 @@ struct SetupArgs {
   uint64_t n[kMaxGeoms];
   uint64_t pid0[kMaxGeoms];
   uint64_t n_norm[kMaxGeoms];
+  int cut_flights;   // no flight runs through periodic faces (GeoRun::unfold stays 0)
 };
 
 int sm_count();

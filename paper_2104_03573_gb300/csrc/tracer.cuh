@@ -70,9 +70,6 @@ struct RunCfg {
   int tail_max;         // FP32 steady tracer: the tail's draw slots serve warps with at most
                         // this many particles in flight once the work counter has run out (0: off)
   int fused;            // FP32 gradient: the forward tallies and the gradient in one pass
-  // forward pass of a two-pass gradient: flights stop at periodic faces, as
-  // the replay's do (the rounding of a flight's tally depends on its cuts)
-  int no_unfold;
   // particle indices a warp takes at once (WarpRun), a multiple of 32; set by
   // take_chunk() at the launch from the most a warp takes
   unsigned take_chunk;
@@ -1411,7 +1408,7 @@ __device__ __forceinline__ void region_steady(const Particle<R>& p, R seg, const
 // flights are cut.
 template <class Grad>
 __device__ __forceinline__ unsigned unfold_mask(const GeoRun& g, const RunCfg& C) {
-  if (Grad::on || C.no_unfold) return 0u;
+  if (Grad::on) return 0u;
   return (unsigned)g.unfold & ~(C.n_cells > 0 ? (1u << C.cell_axis) : 0u);
 }
 
