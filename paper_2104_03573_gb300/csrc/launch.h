@@ -94,9 +94,9 @@ struct MatBuild {
 
 cudaError_t launch_material_build(const MatBuild& b, cudaStream_t s);
 
-// Particle indices a warp takes at once: at most `most` (one returning atomic
-// per chunk), and about four chunks per warp of the grid, so that a run of few
-// particles spreads over all of them.  Runs of 256 left 16 warps of 3648 with
+// Particle indices a warp takes at once: a multiple of 32, at most `most` (one
+// returning atomic per chunk), and about four chunks per warp of the grid, so
+// that a run of few particles spreads over all of them.  Runs of 256 left 16 warps of 3648 with
 // work at 4096 particles and 391 at 100 000 (gray slab of 1e5 particles: main
 // kernel 212 us, 35 us with runs of 32 and the block's sums in BlockAcct).
 inline unsigned take_chunk(uint64_t total, uint64_t warps, unsigned most) {
@@ -108,8 +108,10 @@ inline unsigned take_chunk(uint64_t total, uint64_t warps, unsigned most) {
 // fewer branches its events take one after the other.  FP64: one warp per
 // scheduler, whose pipe it fills (pore film, 2000 particles 1.80 -> 1.62 ms;
 // hot spot, 5000 2.01 -> 1.65; beyond 32 x 4 warps per SM 20 000 particles take
-// 8.65 ms either way).  FP32: all warps, 4 lanes, or 16 where a warp with 8
-// left parks them (gray slab, 4096 particles 110 -> 107 us).
+// 8.65 ms either way).  FP32: all warps, 4 lanes at least, also where the warps
+// park what they hold at once (us with shares of 16, 8 and 4: gray slab of 4096
+// particles 116, 108, 109; silicon-like slab of 4096 1422, 1200, 1199; pore
+// film of 2000 183, 170, 170; 20 films of 100 each 201, 154, 152).
 inline unsigned take_chunk(uint64_t total, uint64_t warps, unsigned most, uint64_t spread, unsigned least) {
   if (total > 32 * spread) return take_chunk(total, warps, most);
   const uint64_t c = (total + spread - 1) / spread;

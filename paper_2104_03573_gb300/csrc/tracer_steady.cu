@@ -1216,8 +1216,7 @@ cudaError_t launch_f32_kernel(const GeoRun* geos, const uint64_t* offs, const Ma
   // to another geometry flushes its sums (20 films of 180-9000 nm, 8e5
   // particles: 2.37 ms with four chunks per warp, 0.90 with one; 14e6 in 64
   // films 23.1 and 22.9)
-  if (C.n_geoms > 1) R.take_chunk = take_chunk(C.total, (warps + 3) / 4, C.take_chunk, warps, 16u);
-  else R.take_chunk = take_chunk(C.total, warps, C.take_chunk, warps, MODE == 0 ? 4u : 16u);
+  R.take_chunk = take_chunk(C.total, C.n_geoms > 1 ? (warps + 3) / 4 : warps, C.take_chunk, warps, 4u);
   kern<<<sm_count() * b, TPB, S.bytes, s>>>(geos, offs, M, R, A, S);
   return cudaGetLastError();
 }
