@@ -168,7 +168,7 @@ mcbte_status mcbte_geometry_create(const mcbte_geometry_desc* desc, mcbte_geomet
 void mcbte_geometry_destroy(mcbte_geometry* g);
 
 /* ------------------------------------------------------------------ runs */
-enum { MCBTE_FP64_PLAIN = 0,      /* one thread per particle, FP64 throughout  */
+enum { MCBTE_FP64_PLAIN = 0,      /* FP64 throughout                            */
        MCBTE_FP32_TRACE = 1 };    /* persistent FP32 tracer, FP64 tallies      */
 
 /* stats[] layout of every run (per geometry for steady runs) */
@@ -316,9 +316,11 @@ typedef struct {
   double time_budget_s;
   void* trace_event_start;     /* optional cudaEvent_t pair around the tracing kernel     */
   void* trace_event_stop;
-  int window_times;            /* FP32 path: measurement times per time window; 0 picks the
-                                  largest window whose tally slice fits a third of the L2;
-                                  >= n_times traces in one pass (no state buffer)           */
+  int window_times;            /* FP32 path: measurement times per time window; 0 picks one
+                                  window for snapshots on the box grid, and for bin averages
+                                  and detector regions the largest window whose tally slice
+                                  fits a third of the L2; >= n_times traces in one pass (no
+                                  state buffer)                                             */
   int n_regions;               /* detector regions (Sec. 4.5, Measure_region), 0..MCBTE_MAX_REGIONS;
                                   0: the whole box split by grid                            */
   const double* regions;       /* HOST [n_regions][6] xmin, xmax, ymin, ymax, zmin, zmax (m)  */

@@ -320,7 +320,7 @@ class TransientConfig:
     blocks_per_sm: int = 0
     time_budget_s: float = 0.0
     trace_events: Optional[tuple] = None
-    window_times: int = 0                    # measurement times per time window (0: sized to the L2)
+    window_times: int = 0                    # measurement times per time window (0: automatic)
     regions: Sequence = ()                   # ((xmin, xmax, ymin, ymax, zmin, zmax) m, (nx, ny, nz)) per region
     time_average: bool = False               # averages over [t_{m-1}, t_m) instead of snapshots at t_m
 

@@ -22,11 +22,13 @@ LIB = os.path.join(HERE, "libmcbte.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 # (source, extra flags, fused multiply-add allowed)
-# FP32 tracers: denormals flushed.  Every quantity they hold (nm, ps, direction
-# cosines, factors) is 0 or far above 1e-38, so the results are the same bits,
-# and the hardware approximations (reciprocal, square roots, logarithm, sines)
-# come without the instructions that handle denormals (41-44 -> 18 cycles each
-# on a lone particle's chain).
+# FP32 tracers: denormals flushed.  For lengths, free paths and velocities from
+# 1e-30 to 1e30 nm and nm/ps every quantity they hold (nm, ps, direction cosines,
+# factors) is 0 or above 1e-38, so the results are the same bits, and the
+# hardware approximations (reciprocal, square roots, logarithm, sines) come
+# without the instructions that handle denormals (41-44 -> 18 cycles each on a
+# lone particle's chain).  Nothing checks that range: beyond it float itself
+# ends (1/v of a velocity below 1e-38 nm/ps is infinite either way).
 FTZ = "--ftz=true"
 UNITS = [
     ("tables.cu", [], False),

@@ -1070,7 +1070,7 @@ mcbte_status mcbte_run_transient(const mcbte_material* m, const mcbte_geometry* 
   A.events_pp = host_out ? w.events_pp : out->events_pp;
   A.tstate = w.tstate;
   if (p->trace_event_start) RUN_TRY(record_trace_event(p->trace_event_start, s));
-  // one launch per time window (a single one unless the FP32 tally exceeds the L2 budget)
+  // one launch per time window
   for (int k = 0; k < n_win; ++k) {
     C.win_first = k == 0;
     C.win_last = k == n_win - 1;

@@ -72,7 +72,7 @@ cudaError_t launch_finalize_transient(const GeoRun* geos, const MatView& M, cons
                                       double* tally, double* stats, size_t n_cells_total, bool fixed,
                                       cudaStream_t s);
 
-// Material table build (FP64): per-bin kernel + one thread per alias table.
+// Material table build (FP64): per-bin kernel + one block per alias table.
 struct MatBuild {
   int n;
   const double *omega, *v, *tau, *C_in, *D, *domega;

@@ -4,7 +4,7 @@
 // derivative of the Bose-Einstein mode energy, Eq. Nbin), or C_i given
 // (format 2); emission weights C v (Eqs. iso_flux, grad_flux_sim), C
 // (Eq. Nbin) and relaxation weights C / tau (Eq. n_scatt); unit conversion
-// to nm / ps.  Then one thread per table builds Walker's alias table with
+// to nm / ps.  Then one block per table builds Walker's alias table with
 // Vose's two work lists (filled in increasing bin order, popped from the
 // back), so the table is a deterministic function of the weights.
 #include "launch.h"
@@ -75,12 +75,15 @@ __device__ __forceinline__ bool below_one(double x) { return __double_as_longlon
 // blockIdx.x = 0..2 builds alias table k (weights C v, C, C / tau);
 // blockIdx.x = 3 forms the sums and the relaxation pmf.  The sums and the
 // walk through Vose's lists are sequential (bin order, so the table is a fixed
-// function of the weights), and their dependent FP64 additions are the
-// kernel's time: one per bin for a sum (the three sums on three warps), two
-// per bin for the walk, which keeps the bin it fills in registers and reads
-// the next ones ahead.  The lists and the per-bin arithmetic are the block's.
-// With `smem` the work arrays live in shared memory, else in the global
-// scratch.  3000 bins: 774 us with the lists and the walk read step by step.
+// function of the weights), and their chains are the kernel's time: one FP64
+// addition per bin for a sum (the three sums on three warps), and the walk's
+// steps, which keep the bin they fill in registers and read the next ones
+// ahead.  The lists and the per-bin arithmetic are the block's.  With `smem`
+// the work arrays live in shared memory, else in the global scratch.
+// 3000 bins: 774 us with the lists and the walk read step by step, now 549: of
+// 1.13e6 cycles 0.22e6 the sum (75 a bin), 0.88e6 the walk (293 a step: two
+// additions, a branch on their result, and the list and bin read for the step
+// after the next), 0.03e6 all the rest.
 __global__ void k_alias(MatBuild b, int smem) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ double s_tot;

@@ -67,10 +67,11 @@ __device__ __forceinline__ float d2_lone(const LoneArgs& A, int bin, float E2) {
   return isinf(lam2) ? Num<float>::inf() : lam2 * E2;
 }
 
-// Reciprocal by the hardware's approximation.  a * rcp_hw(b) has the bits of
-// __fdividef(a, b) for every b in the normal range (2^33 random pairs over
-// exponents -60 to 57 compared), so a quotient can be split where b is known
-// before a.
+// Reciprocal by the hardware's approximation.  a * rcp_hw(b) had the bits of
+// __fdividef(a, b) in 2^33 random pairs with exponents -60 to 57, so a quotient
+// can be split where b is known before a.  (The divisors here lie in that
+// range: direction components, free paths and the pore's root in nm.  Beyond
+// 2^126 __fdividef gives 0.)
 __device__ __forceinline__ float rcp_hw(float b) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
@@ -356,9 +357,15 @@ __device__ __forceinline__ float film_events(const GeoRun& g, unsigned um) {
   return 1.0f + LW * rcp_hw(LA) + LW * rcp_hw(LB);
 }
 // A round of draws ahead costs a warp about as much as four flights that draw
-// inline, so thick films, whose slots end before that, take no slots.
+// inline, so thick films, whose slots end before that, take no slots (silicon,
+// 1e5 particles, us with the line at 1, 2, 4, 8 and 16 flights: film of 300 nm
+// 613, 617, 612, 622, 726; 600 nm 530, 520, 519, 490, 485; 1000 nm 434, 434,
+// 369, 365, 366; 20 films of 10 to 10 000 nm 4284, 4284, 4284, 4733, 4728).  The
+// warp decides for all it holds, by most of its live particles.
 constexpr float kInlineFlights = 4.0f;
-constexpr float kInlineRound = 32.0f;   // flights of a round without slots (then the warp votes again)
+// Flights of a round without slots, then the warp votes again (film of 600 nm
+// with 8, 32 and 128: 542, 519, 512 us; of 150 nm 888, 894, 924).
+constexpr float kInlineRound = 32.0f;
 
 // The tail loop of a film: a box without pore or walls whose flights run
 // through the two periodic axes (forward run without cell tallies or extended

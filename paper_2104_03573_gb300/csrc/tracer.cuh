@@ -691,7 +691,6 @@ struct TallyFxT {
     }
   }
 };
-using TallyFx = TallyFxT<4>;
 
 // No steady tallies (transient runs).
 struct TallyNone {

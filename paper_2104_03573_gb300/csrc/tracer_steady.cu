@@ -1,8 +1,9 @@
-// Steady-state tracing (Sec. 3.6, Eq. steady_estimate): the FP64 plain
-// kernel (one thread per particle, FP64 throughout) and the persistent FP32
-// kernel (FP32 flights; 64-bit fixed-point tallies privatised in shared
-// memory, reduced to FP64; per-lane refill from a warp-aggregated work
-// counter; alias tables in shared memory), plus the finalisation kernel.
+// Steady-state tracing (Sec. 3.6, Eq. steady_estimate): the persistent FP64
+// plain kernel (FP64 throughout) and the persistent FP32 kernel (FP32 flights;
+// 64-bit fixed-point tallies privatised in shared memory, reduced to FP64;
+// alias tables in shared memory), plus the finalisation kernel.  In both a lane
+// that is done takes its warp's next particle, from the run of indices that the
+// warp holds or takes from the work counter (WarpRun).
 //
 // This file is compiled three times: with MCBTE_F64 (FP64 kernels, no fused
 // multiply-add) and with MCBTE_F32 twice, MCBTE_F32_PART 0 (the FP32 kernels

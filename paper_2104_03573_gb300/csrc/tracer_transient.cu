@@ -1,8 +1,8 @@
 // Transient tracing (Secs. 3.2-3.5): wall sources emit at t0 = R t_max, the
 // initial condition at t0 = 0 (Sec. 3.2); every measurement time inside a
 // particle's life adds its snapshot to the detector grid (Eq. sampling).
-// FP64 plain kernel (one thread per particle) and persistent FP32 kernel
-// (per-lane refill, alias tables in shared memory, FP64 L2 atomics into the
+// Persistent FP64 plain kernel and persistent FP32 kernel (per-lane refill,
+// alias tables in shared memory, 64-bit fixed-point reductions into the
 // [time][cell][T, qx, qy, qz] tally, which is far larger than shared memory).
 #include "launch.h"
 
@@ -368,8 +368,8 @@ __device__ __forceinline__ void warp_bin_averages(int k, float t_end, const Part
 }
 
 // Shared memory: the warps' flight slots (snapshots), the measurement times as
-// float (always), then the relaxation
-// alias records and per-bin constants where the plan has room.
+// float (always), then the relaxation alias records and per-bin constants where
+// the plan has room.
 // TAVG: the run tallies time-bin averages (compiled apart, so that the
 // snapshot variant carries none of that code).
 template <int TPB, bool EXT, bool TAVG>
