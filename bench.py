@@ -17,9 +17,9 @@ Other workloads (`--workload`), same line format:
   nanomesh       the paper's square-pore nanomesh (four internal walls), 1e6
                  particles, N_scat_max 10, separate two-phonon clock
   transient_box  2x2x1 um diffuse box, +1 K Gaussian hot spot, 1e8 particles,
-                 64x64x32 cells x 200 snapshot times (fixed-point L2 reductions
-                 in L2-sized time windows); also reports the reductions' rate
-                 against the library's L2 reduction probe
+                 64x64x32 cells x 200 snapshot times (fixed-point reductions of
+                 whole records, one launch); also reports the reductions' rate
+                 against the bench's probe
   transient_box_avg  the same box with 200 time-bin averages instead of
                  snapshots
   film_batch     64 films 10 nm..10 um in one persistent launch replayed as
@@ -74,12 +74,12 @@ WORKLOADS = {"si_slab": "si_slab_L1um_3000bins", "si_slab_imp": "si_slab_L1um_30
 # draw, state update and tallies: 200 thread-instructions).
 INSTR_PER_EVENT = 200.0
 NCU_INSTR_PER_EVENT = {   # workload: (thread-instructions, warp-instructions) per event
-    "si_slab": (375.9, 19.06),    # 2.488e11 / 1.261e10 instructions over 6.619e8 events
+    "si_slab": (352.9, 18.54),    # 2.336e11 / 1.227e10 instructions over 6.619e8 events
 }
 # DRAM bytes per launch of the FP32 steady tracing kernel on the default
 # workload, from the ncu capture summarised in profiles/ (None until a capture
 # of the current kernel exists).
-TRACE_DRAM_BYTES_PER_LAUNCH = 1_713_152 + 40_448
+TRACE_DRAM_BYTES_PER_LAUNCH = 348_928 + 19_712
 
 
 PROBE_SRC = os.path.join(ROOT, "bench_l2_probe.cu")
@@ -101,8 +101,9 @@ def build_probe(force: bool = False) -> str:
 def load_probe():
     build_probe()
     lib = ctypes.CDLL(PROBE_LIB)
-    lib.bench_l2_reduction_probe.argtypes = [ctypes.c_void_p, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
-    lib.bench_l2_reduction_probe.restype = ctypes.c_int
+    for f in (lib.bench_l2_reduction_probe, lib.bench_l2_record_probe):
+        f.argtypes = [ctypes.c_void_p, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
+        f.restype = ctypes.c_int
     return lib
 
 
@@ -466,22 +467,25 @@ def _workload_setup(name, args, seed_offset, rank=0, world=1):
                                                    None), allow=(LL.OK, LL.WARN_TRUNCATED))
             return st[None, :]
         nt = len(run.t_meas) * run.grid[0] * run.grid[1] * run.grid[2] * 4 * 8
-        # time windows of the FP32 run (the library's automatic choice: the
-        # largest window whose tally slice fits a third of the L2)
+        # time windows of the FP32 run (the library's automatic choice: one for
+        # snapshots on the box grid, for bin averages the largest whose tally
+        # slice fits a third of the L2)
         slice_b = run.grid[0] * run.grid[1] * run.grid[2] * 4 * 8
         l2 = int(getattr(torch.cuda.get_device_properties(torch.cuda.current_device()), "L2_cache_size", 96 << 20))
-        wt = max(1, min(len(run.t_meas), (l2 // 3) // slice_b))
+        wt_l2 = max(1, min(len(run.t_meas), (l2 // 3) // slice_b))
+        wt = wt_l2 if run.time_average else len(run.t_meas)
         windows = -(-len(run.t_meas) // wt)
         desc = ("transient 2x2x1 um diffuse adiabatic box, +1 K Gaussian sigma 100 nm at the top-face centre, "
                 "64x64x32 cells x 200 " + ("10 ps bin averages" if run.time_average else "snapshots (10 ps)")
-                + ", FP32 flights, fixed-point tallies in L2-sized time windows")
+                + ", FP32 flights, fixed-point tallies"
+                + (" in L2-sized time windows" if run.time_average else ", one launch"))
         return dict(mat=mat, geo=geo, run=run, n=run.n, step=step, fp64=fp64, e2e=e2e, d2h=nt + 8 * L.NSTATS,
                     h2d=_material_bytes(mat) + ctypes.sizeof(L.GeometryDesc) + 8 * len(run.t_meas), desc=desc,
                     launches=2 + windows, timer=tm, kernel="k_transient_f32",
                     shape={"threads_per_block": cfg.threads_per_block, "time_windows": windows},
                     kappa=False, kind="transient",
                     # adiabatic box: every particle lives to t_max, so it is sampled at all n_times
-                    tally_ops=run.n * len(run.t_meas), l2_slice_words=wt * slice_b // 8)
+                    tally_ops=run.n * len(run.t_meas), l2_slice_words=wt_l2 * slice_b // 8)
     raise ValueError(name)
 
 
@@ -702,23 +706,26 @@ def t_kern_probe(kern_ms):
 
 
 def l2_reduction_roofline(wk, t_kern):
-    """Snapshot-bound transient runs: the 64-bit L2 reductions the tracing
-    kernels issue per second (4 per snapshot) against the rate the bench's
-    probe (bench_l2_probe.cu) reaches in the same pattern on an array the size of one time
-    window's tally slice (best of 3 timed launches)."""
+    """Tally-bound transient runs: the 64-bit reductions the tracing kernels
+    issue per second (4 per snapshot) against the rate the bench's probe
+    (bench_l2_probe.cu) reaches in the same pattern (whole records for
+    snapshots, word by word for bin averages) on an array that stays in the L2
+    (at most a third of it; best of 3 timed launches): what the L2 takes at
+    most.  A tally larger than the L2 costs DRAM traffic on top."""
     import torch
     from paper_2104_03573_gb300 import _lib as L
     words = int(wk["l2_slice_words"]) // 4 * 4
     slots = torch.zeros(words, dtype=torch.int64, device="cuda")
     groups = 1 << 28
-    lib = load_probe()
+    records = not wk["run"].time_average
+    probe = load_probe().bench_l2_record_probe if records else load_probe().bench_l2_reduction_probe
     s = torch.cuda.current_stream()
-    assert lib.bench_l2_reduction_probe(slots.data_ptr(), words, groups // 16, ctypes.c_void_p(s.cuda_stream)) == 0
+    assert probe(slots.data_ptr(), words, groups // 16, ctypes.c_void_p(s.cuda_stream)) == 0
     best = None
     for _ in range(3):
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(s)
-        assert lib.bench_l2_reduction_probe(slots.data_ptr(), words, groups, ctypes.c_void_p(s.cuda_stream)) == 0
+        assert probe(slots.data_ptr(), words, groups, ctypes.c_void_p(s.cuda_stream)) == 0
         e1.record(s)
         e1.synchronize()
         t = e0.elapsed_time(e1) / 1e3
@@ -726,8 +733,8 @@ def l2_reduction_roofline(wk, t_kern):
     peak = 4.0 * groups / best / 1e9
     achieved = 4.0 * wk["tally_ops"] / t_kern / 1e9
     return {"achieved": achieved, "peak": peak, "unit": "G reductions/s", "frac": achieved / peak,
-            "peak_basis": f"bench_l2_probe.cu: 2^28 groups of 4 64-bit reductions into a "
-                          f"{words * 8 / 2**20:.0f} MiB array (one time window's tally slice), best of 3"}
+            "peak_basis": f"bench_l2_probe.cu: 2^28 {'records' if records else 'groups'} of 4 64-bit reductions into "
+                          f"a {words * 8 / 2**20:.0f} MiB array in the L2, best of 3"}
 
 
 def cpu_baseline(wk, args, target_s=None):
