@@ -29,6 +29,7 @@ int sm_count();
 // events each: 21.9 ms at 16 warps a SM, 17.2 at 8, 16.0 at 6, 15.2 at 4; 2e6
 // particles: 58.9, 54.2, 54.4, 63.0).
 constexpr int kF64Threads = 192;
+constexpr int kF64RegionThreads = 128;   // k_transient_fp64_regions: one warp per scheduler
 inline int f64_blocks(uint64_t total) {
   const uint64_t most = (uint64_t)sm_count();   // a warp on every SM first
   return (int)(total < most ? total : most);

@@ -53,13 +53,17 @@ def test_fp64_steady_refills(n):
 
 @pytest.mark.parametrize("n", EDGES.values(), ids=EDGES.keys())
 @pytest.mark.parametrize("average", [False, True])
+@pytest.mark.parametrize("regions", [False, True])
 @pytest.mark.parametrize("walls", [False, True])
-def test_fp64_transient_refills(walls, average, n):
+def test_fp64_transient_refills(walls, regions, average, n):
     # 20 ps: a few events per particle; a hot spot at the start, or walls that
     # emit over the whole time (a lane's next particle may start before its last)
     wl = W.ballistic_transient_e1(n=n) if walls else W.transient_box_c3(n=n, grid=(4, 3, 5), n_times=6)
     mat, g, run = W.bvk_holland(), wl.geometries[0], wl.run
     run.t_max, run.time_average = 2e-11, average
+    if regions:
+        x, y, z = g.L
+        run.regions = [((0.2 * x, 0.9 * x, 0.1 * y, 0.8 * y, 0.0, 0.7 * z), (2, 3, 1)), ((0.0, x, 0.0, y, 0.0, z), (1, 2, 2))]
     run.t_meas = run.t_max * np.arange(1, 7) / 6
     gg = gpu_transient(mat, g, run, L.FP64_PLAIN, per_particle=True)
     ref = oracle.run_transient(mat, g, run, per_particle=True)
