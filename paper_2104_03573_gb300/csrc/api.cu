@@ -896,9 +896,9 @@ uint64_t transient_detectors(const mcbte_transient_params* p) {
 
 // FP32 transient time windows: measurement times per window.  Automatic
 // choice: the whole run for snapshots on the box grid, whose reductions add
-// whole 32-byte records (hot spot of 1e7 particles, 64 x 64 x 32 cells x 200
-// times, an 839 MB tally: 45.0 ms in one window, 50.5 in 20 of the L2's size;
-// word by word it was 105 against 51.6).  Bin averages and detector regions
+// whole 32-byte records where that pays (hot spot of 1e7 particles, 64 x 64 x 32
+// cells x 200 times, an 839 MB tally: 48 ms in one window, 51 in 20 of the L2's
+// size; word by word 107 against 52).  Bin averages and detector regions
 // add word by word: the largest window whose [times][cells][4] x 8-byte slice
 // of the tally fits a third of the L2.
 int transient_window_times(const mcbte_transient_params* p) {
@@ -915,6 +915,23 @@ int transient_window_times(const mcbte_transient_params* p) {
     wt = fit < 1 ? 1 : (fit > (size_t)p->n_times ? p->n_times : (int)fit);
   }
   return wt < p->n_times ? wt : p->n_times;
+}
+
+// How the FP32 grid snapshots of a launch whose slice of the tally takes
+// `bytes` are added (RunCfg::snap_records).  A tally in the L2 takes single
+// words as fast as records, which cost more instructions (hot spot of 1e7
+// particles, ms by records / words: 6.6 MB 37.1 / 32.6, 52 MB 37.0 / 32.5,
+// 105 MB 44.0 / 41.8), except on the few addresses of a small one (one cell x
+// 100 times 92.8 / 410.7; 0.16 MB 37.1 / 40.9; 0.8 MB 37.1 / 36.7).  Beyond the L2
+// every word is a transaction of its own, so a step with many snapshots adds
+// records (records / words / by the step: 419 MB of 100 times 37.3 / 35.8 / 35.2,
+// 839 MB of 200 times 48.3 / 107.4 / 44.1, 1678 MB of 50 times 37.0 / 31.6 / 32.4).
+int transient_snap_records(size_t bytes) {
+  if (bytes < ((size_t)1 << 19)) return 2;
+  int dev = 0, l2 = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+    l2 = 0;
+  return bytes <= (size_t)l2 ? 0 : 1;
 }
 
 TransientWs layout_transient(char* base, size_t snap_len, int n_times, bool host_out, bool want_ev, uint64_t total,
@@ -1047,6 +1064,7 @@ mcbte_status mcbte_run_transient(const mcbte_material* m, const mcbte_geometry* 
   C.t_max_ps = p->t_max * 1e12;
   C.ext = uses_ext(m, g->host) ? 1 : 0;
   C.n_times = p->n_times;
+  C.snap_records = transient_snap_records((size_t)wt * ncell * 4 * sizeof(double));
   C.t_meas_ps = w.t_meas_ps;
   for (int k = 0; k < 3; ++k) C.grid[k] = p->grid[k];
   // detector regions, derived on the host with the CPU reference's arithmetic;

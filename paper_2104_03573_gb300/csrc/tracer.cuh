@@ -70,6 +70,9 @@ struct RunCfg {
   int tail_max;         // FP32 steady tracer: the tail's draw slots serve warps with at most
                         // this many particles in flight once the work counter has run out (0: off)
   int fused;            // FP32 gradient: the forward tallies and the gradient in one pass
+  // FP32 grid snapshots added as whole records by quads of lanes: 2 always,
+  // 1 where a warp's step has many, 0 never (word by word)
+  int snap_records;
   // particle indices a warp takes at once (WarpRun); set by take_chunk() at the
   // launch from the most a warp takes: a multiple of 32, or an equal share of a
   // run that the grid's warps hold whole (then none is taken later)

@@ -71,6 +71,81 @@ struct WarpAcct {
   }
 };
 
+// The same by lanes: each adds its own finished particles, and the warp's lanes
+// are summed at the kernel's end.  For the FP32 kernel, whose steps are too
+// short for WarpAcct's votes (1e7 particles, a tally of 52 MB: 38.0 ms with the
+// votes, 37.0 without); kept in local memory (acct_of), since a lane touches it
+// once per particle and the event loop needs the registers.
+struct LaneAcct {
+  unsigned long long ev;
+  unsigned traced, trunc, maxev, absorbed;
+  int s_emit, s_abs;
+
+  __device__ __forceinline__ void reset() {
+    ev = 0ull;
+    traced = trunc = maxev = absorbed = 0u;
+    s_emit = s_abs = 0;
+  }
+  __device__ __forceinline__ void end(int out, uint32_t e, float s) {
+    const unsigned nev = e + 1u;
+    const int sgn = s > 0.0f ? 1 : -1;
+    ev += nev;
+    maxev = nev > maxev ? nev : maxev;
+    traced += 1u;
+    trunc += out == STEP_TRUNCATED ? 1u : 0u;
+    s_emit += sgn;
+    if (out == STEP_ABSORBED) {
+      absorbed += 1u;
+      s_abs += sgn;
+    }
+  }
+  // called by all 32 lanes
+  __device__ __forceinline__ void flush(unsigned lane, const Acc& A) const {
+    constexpr unsigned kAll = 0xffffffffu;
+    unsigned long long ev_w = ev, tr = traced;
+    long long se = s_emit, sa = s_abs;
+    const unsigned tc = __reduce_add_sync(kAll, trunc), ab = __reduce_add_sync(kAll, absorbed);
+    const unsigned mx = __reduce_max_sync(kAll, maxev);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      ev_w += __shfl_xor_sync(kAll, ev_w, o);
+      tr += __shfl_xor_sync(kAll, tr, o);
+      se += __shfl_xor_sync(kAll, se, o);
+      sa += __shfl_xor_sync(kAll, sa, o);
+    }
+    if (lane != 0u || tr == 0ull) return;
+    unsigned long long* cnt = A.cnt + sum_copy() * 4;
+    double* dsc = A.dsc + sum_copy() * 8;
+    atomicAdd(cnt + 0, ev_w);
+    if (tc) atomicAdd(cnt + 1, (unsigned long long)tc);
+    atomicMax(cnt + 2, (unsigned long long)mx);
+    atomicAdd(cnt + 3, tr);
+    atomicAdd(dsc + 2, (double)se);
+    if (ab) {
+      atomicAdd(dsc + 3, (double)sa);
+      atomicAdd(dsc + 7, (double)ab);
+    }
+  }
+};
+
+// One finished particle added at once: bin averages, whose kernel has no
+// register left for a lane's own counters (1e7 particles: 191.5 ms with them,
+// 187.8 without) and whose particles are long.
+__device__ __forceinline__ void transient_finish(const Particle<float>& p, int out, const Acc& A) {
+  const unsigned long long nev = (unsigned long long)p.e + 1ull;
+  unsigned long long* cnt = A.cnt + sum_copy() * 4;
+  double* dsc = A.dsc + sum_copy() * 8;
+  atomicAdd(cnt + 0, nev);
+  if (out == STEP_TRUNCATED) atomicAdd(cnt + 1, 1ull);
+  atomicMax(cnt + 2, nev);
+  atomicAdd(cnt + 3, 1ull);
+  atomicAdd(dsc + 2, (double)p.s);
+  if (out == STEP_ABSORBED) {
+    atomicAdd(dsc + 3, (double)p.s);
+    atomicAdd(dsc + 7, 1.0);
+  }
+}
+
 #if MCBTE_F64
 // Persistent, like k_steady_fp64: 32 particles emitted at a time, a lane that
 // is done refills.
@@ -278,13 +353,17 @@ struct FlightSlots {
 // of the flight that starts at p.x at time p.t); a lane's count depends on
 // its flight's length, so a per-lane loop would leave most lanes idle while
 // the longest flights sample.  Here the warp's k_1 + ... + k_32 snapshots are
-// taken 32 at a time.  The flights that have any are written to `fs`, side by
-// side in lane order; where each begins among the 32 of a round is one bit of
-// a mask, so a lane finds its snapshot's flight by a population count.  (A
-// bisection of the prefix sums and ten shuffles of the owner's state took its
-// place before: hot spot of 1e7 particles and 200 snapshots 49.2 ms, now
-// 45.0.)  Every lane of the warp must call this (k = 0 for idle lanes).
-// The arithmetic per snapshot is the per-lane loop's (Eq. sampling, Sec. 3.4).
+// taken 32 at a time.  Every lane of the warp must call this (k = 0 for idle
+// lanes).  The arithmetic per snapshot is the per-lane loop's (Eq. sampling,
+// Sec. 3.4).
+//
+// Whole records (C.snap_records: 2 always, 1 where the step has 24 snapshots
+// or more): the flights that have snapshots are written to `fs`, side by side in
+// lane order; where each begins among the 32 of a round is one bit of a mask,
+// so a lane finds its snapshot's flight by a population count, and the quads
+// add their records (red_records).  Fewer reductions, more instructions.
+// Word by word: a bisection of the prefix sums and shuffles of the owner's
+// state, four reductions per lane.  transient_snap_records() chooses.
 __device__ __forceinline__ void warp_snapshots(int k, const Particle<float>& p, const float* tmeas, const float* cinv,
                                                const RunCfg& C, double* snap, FlightSlots& fs) {
   constexpr unsigned kAll = 0xffffffffu;
@@ -298,6 +377,50 @@ __device__ __forceinline__ void warp_snapshots(int k, const Particle<float>& p, 
     if (lane >= o) incl += y;
   }
   const int total = __shfl_sync(kAll, incl, 31);
+  const int nx = C.grid[0], ny = C.grid[1], nz = C.grid[2];
+  const size_t ncell = (size_t)nx * ny * nz;
+  if (C.snap_records == 0 || (C.snap_records == 1 && total < 24)) {
+    for (int base = 0; base < total; base += 32) {
+      const int j = base + lane;
+      // owner: the first lane whose inclusive sum exceeds j (always in 0..31)
+      int own = 0;
+#pragma unroll
+      for (int st = 16; st >= 1; st >>= 1) {
+        const int v = __shfl_sync(kAll, incl, own + st - 1);
+        if (v <= j) own += st;
+      }
+      const int first = __shfl_sync(kAll, incl - k, own);
+      const int mi0 = __shfl_sync(kAll, p.mi, own);
+      const float x0 = __shfl_sync(kAll, p.x[0], own), x1 = __shfl_sync(kAll, p.x[1], own),
+                  x2 = __shfl_sync(kAll, p.x[2], own);
+      const float u0 = __shfl_sync(kAll, p.u[0], own), u1 = __shfl_sync(kAll, p.u[1], own),
+                  u2 = __shfl_sync(kAll, p.u[2], own);
+      const float t0 = __shfl_sync(kAll, p.t, own), v = __shfl_sync(kAll, p.v, own), s = __shfl_sync(kAll, p.s, own);
+      if (j < total) {
+        const int m = mi0 + (j - first);
+        const float dist = v * (tmeas[m] - t0);
+        const float pm0 = x0 + dist * u0, pm1 = x1 + dist * u1, pm2 = x2 + dist * u2;
+        const int ix = min(max((int)floorf(pm0 * cinv[0]), 0), nx - 1);
+        const int iy = min(max((int)floorf(pm1 * cinv[1]), 0), ny - 1);
+        const int iz = min(max((int)floorf(pm2 * cinv[2]), 0), nz - 1);
+        long long* q = reinterpret_cast<long long*>(snap) + ((size_t)m * ncell + ((size_t)iz * ny + iy) * nx + ix) * 4;
+        const float sv = s * v;
+        red_s64(q + 0, s > 0.0f ? 1ll : -1ll);
+        if (v < 1024.0f) {
+          // |s v u_a| <= v (1 + rounding): below 2^30 in fixed point, so the
+          // 32-bit conversion gives the value fx gives
+          red_s64(q + 1, (long long)__float2int_rn((sv * u0) * kFx));
+          red_s64(q + 2, (long long)__float2int_rn((sv * u1) * kFx));
+          red_s64(q + 3, (long long)__float2int_rn((sv * u2) * kFx));
+        } else {
+          red_s64(q + 1, fx(sv * u0));
+          red_s64(q + 2, fx(sv * u1));
+          red_s64(q + 3, fx(sv * u2));
+        }
+      }
+    }
+    return;
+  }
   const int excl = incl - k;
   if (k > 0) {
     const int r = __popc(some & ((1u << lane) - 1u));
@@ -306,8 +429,6 @@ __device__ __forceinline__ void warp_snapshots(int k, const Particle<float>& p, 
     fs.first[r] = p.mi - excl;
   }
   __syncwarp();
-  const int nx = C.grid[0], ny = C.grid[1], nz = C.grid[2];
-  const size_t ncell = (size_t)nx * ny * nz;
   const bool narrow = ncell * (size_t)C.n_times < (size_t)kNoRec;
   int before = -1;   // flights that begin before this round, less one
   for (int base = 0; base < total; base += 32) {
@@ -459,7 +580,13 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
   Particle<float> p;
   p.e = 0u;
   p.s = 0.0f;
-  WarpAcct acct;
+  LaneAcct acct;
+  acct.reset();
+  auto acct_of = [&]() -> LaneAcct* {
+    LaneAcct* q = &acct;
+    asm volatile("" : "+l"(q) : : "memory");   // (no instruction: hides where q points)
+    return q;
+  };
   bool alive = false;
   bool drained = false;   // as in the steady tracer: idle lanes stay until the warp is drained
   uint64_t idx = 0;
@@ -522,7 +649,6 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
       }
       if constexpr (TAVG) warp_bin_averages(k, t_end, p, tmeas, C, A.snap);
       else warp_snapshots(k, p, tmeas, cinv, C, A.snap, *slots);
-      bool ended = false;
       if (alive) {
         if (out == STEP_ALIVE) {
           if constexpr (TAVG) p.mi = mi_next;
@@ -543,7 +669,8 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           out = STEP_TRUNCATED;
         }
         if (out != STEP_ALIVE) {
-          ended = true;
+          if constexpr (TAVG) transient_finish(p, out, A);
+          else acct_of()->end(out, p.e, p.s);
           alive = false;
           if (A.events_pp) A.events_pp[idx] = p.e + 1u;
           if (!C.win_last) mark_done(A.tstate, idx);
@@ -552,9 +679,8 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           alive = false;
         }
       }
-      acct.add(ended, out, p.e, p.s, lane);
     }
-    acct.flush(lane, A);
+    if constexpr (!TAVG) acct_of()->flush(lane, A);
     return;
   }
   // snapshots into detector regions: the per-lane loop
@@ -581,7 +707,6 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
         }
       }
       int out = STEP_ALIVE;
-      bool ended = false;
       if (alive) {
         out = step_transient<float, EXT>(p, G, M, relax, binf, C, key.x, key.y, A.snap, tmeas, cinv);
         if (out == STEP_ALIVE && (p.e & 255u) == 0u && globaltimer_ns() > deadline) {
@@ -589,7 +714,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           out = STEP_TRUNCATED;
         }
         if (out != STEP_ALIVE) {
-          ended = true;
+          acct_of()->end(out, p.e, p.s);
           alive = false;
           if (A.events_pp) A.events_pp[idx] = p.e + 1u;
           if (!C.win_last) mark_done(A.tstate, idx);
@@ -599,9 +724,8 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           alive = false;
         }
       }
-      acct.add(ended, out, p.e, p.s, lane);
     }
-    acct.flush(lane, A);
+    acct_of()->flush(lane, A);
   }
 }
 
