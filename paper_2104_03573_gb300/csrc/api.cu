@@ -922,12 +922,13 @@ int transient_window_times(const mcbte_transient_params* p) {
 // words as fast as records, which cost more instructions (hot spot of 1e7
 // particles, ms by records / words: 6.6 MB 37.1 / 32.6, 52 MB 37.0 / 32.5,
 // 105 MB 44.0 / 41.8), except on the few addresses of a small one (one cell x
-// 100 times 92.8 / 410.7; 0.16 MB 37.1 / 40.9; 0.8 MB 37.1 / 36.7).  Beyond the L2
-// every word is a transaction of its own, so a step with many snapshots adds
-// records (records / words / by the step: 419 MB of 100 times 37.3 / 35.8 / 35.2,
-// 839 MB of 200 times 48.3 / 107.4 / 44.1, 1678 MB of 50 times 37.0 / 31.6 / 32.4).
+// 100 times 92.8 / 410.7; 0.16 MB 37.1 / 40.9; 0.8 MB 36.7 / 35.5, of 1.5e5
+// particles 1.40 / 1.66).  Beyond the L2 every word is a transaction of its own,
+// so a step with many snapshots adds records (records / words / by the step:
+// 210 MB of 50 times 36.1 / 30.6 / 31.4, 419 MB of 100 37.3 / 35.8 / 34.6, 839 MB of
+// 200 48.3 / 107.4 / 48.5, 1678 MB of 50 37.0 / 31.6 / 32.3).
 int transient_snap_records(size_t bytes) {
-  if (bytes < ((size_t)1 << 19)) return 2;
+  if (bytes < ((size_t)1 << 20)) return 2;
   int dev = 0, l2 = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
     l2 = 0;

@@ -71,59 +71,46 @@ struct WarpAcct {
   }
 };
 
-// The same by lanes: each adds its own finished particles, and the warp's lanes
-// are summed at the kernel's end.  For the FP32 kernel, whose steps are too
-// short for WarpAcct's votes (1e7 particles, a tally of 52 MB: 38.0 ms with the
-// votes, 37.0 without); kept in local memory (acct_of), since a lane touches it
-// once per particle and the event loop needs the registers.
-struct LaneAcct {
+// The same in shared memory, added to by the lanes whose particles end.  For
+// the FP32 kernel, whose steps are too short for WarpAcct's votes and whose
+// threads have no registers for counters of their own (1e7 particles with the
+// two-phonon clock: 116.1 ms with votes, 113.4 with a thread's counters in local
+// memory, 110.5 here with the run of indices beside them).
+struct SharedAcct {
   unsigned long long ev;
-  unsigned traced, trunc, maxev, absorbed;
-  int s_emit, s_abs;
+  unsigned traced, trunc, maxev, positive, absorbed, positive_absorbed;
 
+  // by one lane of the warp
   __device__ __forceinline__ void reset() {
     ev = 0ull;
-    traced = trunc = maxev = absorbed = 0u;
-    s_emit = s_abs = 0;
+    traced = trunc = maxev = positive = absorbed = positive_absorbed = 0u;
   }
   __device__ __forceinline__ void end(int out, uint32_t e, float s) {
     const unsigned nev = e + 1u;
-    const int sgn = s > 0.0f ? 1 : -1;
-    ev += nev;
-    maxev = nev > maxev ? nev : maxev;
-    traced += 1u;
-    trunc += out == STEP_TRUNCATED ? 1u : 0u;
-    s_emit += sgn;
+    atomicAdd(&ev, (unsigned long long)nev);
+    atomicAdd(&traced, 1u);
+    atomicMax(&maxev, nev);
+    if (s > 0.0f) atomicAdd(&positive, 1u);
+    if (out == STEP_TRUNCATED) atomicAdd(&trunc, 1u);
     if (out == STEP_ABSORBED) {
-      absorbed += 1u;
-      s_abs += sgn;
+      atomicAdd(&absorbed, 1u);
+      if (s > 0.0f) atomicAdd(&positive_absorbed, 1u);
     }
   }
-  // called by all 32 lanes
+  // called by all lanes of the warp
   __device__ __forceinline__ void flush(unsigned lane, const Acc& A) const {
-    constexpr unsigned kAll = 0xffffffffu;
-    unsigned long long ev_w = ev, tr = traced;
-    long long se = s_emit, sa = s_abs;
-    const unsigned tc = __reduce_add_sync(kAll, trunc), ab = __reduce_add_sync(kAll, absorbed);
-    const unsigned mx = __reduce_max_sync(kAll, maxev);
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-      ev_w += __shfl_xor_sync(kAll, ev_w, o);
-      tr += __shfl_xor_sync(kAll, tr, o);
-      se += __shfl_xor_sync(kAll, se, o);
-      sa += __shfl_xor_sync(kAll, sa, o);
-    }
-    if (lane != 0u || tr == 0ull) return;
+    __syncwarp();
+    if (lane != 0u || traced == 0u) return;
     unsigned long long* cnt = A.cnt + sum_copy() * 4;
     double* dsc = A.dsc + sum_copy() * 8;
-    atomicAdd(cnt + 0, ev_w);
-    if (tc) atomicAdd(cnt + 1, (unsigned long long)tc);
-    atomicMax(cnt + 2, (unsigned long long)mx);
-    atomicAdd(cnt + 3, tr);
-    atomicAdd(dsc + 2, (double)se);
-    if (ab) {
-      atomicAdd(dsc + 3, (double)sa);
-      atomicAdd(dsc + 7, (double)ab);
+    atomicAdd(cnt + 0, ev);
+    if (trunc) atomicAdd(cnt + 1, (unsigned long long)trunc);
+    atomicMax(cnt + 2, (unsigned long long)maxev);
+    atomicAdd(cnt + 3, (unsigned long long)traced);
+    atomicAdd(dsc + 2, (double)(2ll * positive - (long long)traced));
+    if (absorbed) {
+      atomicAdd(dsc + 3, (double)(2ll * positive_absorbed - (long long)absorbed));
+      atomicAdd(dsc + 7, (double)absorbed);
     }
   }
 };
@@ -575,18 +562,29 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
   const uint64_t deadline = *C.t0 + C.budget_ns;
   const unsigned lane = threadIdx.x & 31u;
   const uint2 key = run_key(C);
-  WarpRun run;   // the warp's particle indices not yet handed out
-  run.start(C.take_chunk, C.total, deadline, A.flags);
+  // the warp's particle indices not yet handed out
+  __shared__ WarpRun s_run[TPB / 32];
+  {
+    WarpRun r;
+    r.start(C.take_chunk, C.total, deadline, A.flags);
+    if (lane == 0) s_run[threadIdx.x >> 5] = r;
+    __syncwarp();
+  }
+  auto take = [&](unsigned need) -> uint64_t {
+    WarpRun r = s_run[threadIdx.x >> 5];
+    __syncwarp();
+    const uint64_t k = r.take(need, lane, A.work, C.total, deadline, A.flags);
+    if (lane == 0) s_run[threadIdx.x >> 5] = r;
+    __syncwarp();
+    return k;
+  };
   Particle<float> p;
   p.e = 0u;
   p.s = 0.0f;
-  LaneAcct acct;
-  acct.reset();
-  auto acct_of = [&]() -> LaneAcct* {
-    LaneAcct* q = &acct;
-    asm volatile("" : "+l"(q) : : "memory");   // (no instruction: hides where q points)
-    return q;
-  };
+  __shared__ SharedAcct s_acct[TAVG ? 1 : TPB / 32];
+  SharedAcct& acct = s_acct[TAVG ? 0 : threadIdx.x >> 5];
+  if (!TAVG && lane == 0u) acct.reset();
+  __syncwarp();
   bool alive = false;
   bool drained = false;   // as in the steady tracer: idle lanes stay until the warp is drained
   uint64_t idx = 0;
@@ -600,7 +598,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
       if (__all_sync(kAll, drained)) break;
       const unsigned need = __ballot_sync(kAll, !alive && !drained);
       if (need) {
-        const uint64_t k = run.take(need, lane, A.work, C.total, deadline, A.flags);
+        const uint64_t k = take(need);
         if (!alive && !drained) {
           idx = k;
           if (idx >= C.total || (*(volatile int*)A.flags & 1)) {
@@ -670,7 +668,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
         }
         if (out != STEP_ALIVE) {
           if constexpr (TAVG) transient_finish(p, out, A);
-          else acct_of()->end(out, p.e, p.s);
+          else acct.end(out, p.e, p.s);
           alive = false;
           if (A.events_pp) A.events_pp[idx] = p.e + 1u;
           if (!C.win_last) mark_done(A.tstate, idx);
@@ -680,7 +678,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
         }
       }
     }
-    if constexpr (!TAVG) acct_of()->flush(lane, A);
+    if constexpr (!TAVG) acct.flush(lane, A);
     return;
   }
   // snapshots into detector regions: the per-lane loop
@@ -689,7 +687,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
       if (__all_sync(kAll, drained)) break;
       const unsigned need = __ballot_sync(kAll, !alive && !drained);
       if (need) {
-        const uint64_t k = run.take(need, lane, A.work, C.total, deadline, A.flags);
+        const uint64_t k = take(need);
         if (!alive && !drained) {
           idx = k;
           if (idx >= C.total || (*(volatile int*)A.flags & 1)) {
@@ -714,7 +712,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
           out = STEP_TRUNCATED;
         }
         if (out != STEP_ALIVE) {
-          acct_of()->end(out, p.e, p.s);
+          acct.end(out, p.e, p.s);
           alive = false;
           if (A.events_pp) A.events_pp[idx] = p.e + 1u;
           if (!C.win_last) mark_done(A.tstate, idx);
@@ -725,7 +723,7 @@ __global__ void __launch_bounds__(TPB, 1) k_transient_f32(const GeoRun* __restri
         }
       }
     }
-    acct_of()->flush(lane, A);
+    acct.flush(lane, A);
   }
 }
 
