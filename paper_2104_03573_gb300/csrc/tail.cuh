@@ -398,6 +398,9 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
     cq = fx_lone((s * db) * sel3(p.u, T.ta));
   };
   aim();
+  // the flight ahead runs from wall to wall (its length and tally then stay
+  // under a specular reflection, in every bit)
+  bool full = p.x[W] == (up ? 0.0f : LW);
   // Flights from wall to wall that do not relax, in a loop of their own with
   // the next draws read ahead.  An unsigned comparison of the bits takes
   // 0 <= x < L in one test; a flight past one periodic face is folded here
@@ -413,7 +416,7 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
       uint32_t e = p.e;
       float x = p.x[A], y = p.x[B], ua = p.u[A], ub = p.u[B], l0 = fabsf(p.u[W]), dr = p.d_rel;
       long long X = p.Xq;
-      bool full = false;   // the flight ahead starts at a wall
+      bool moved = false;
       while (e < e_lim) {
         const DrawLean* d = slot0 + (e - e0);
         float4 nx = d->film_flight();
@@ -464,10 +467,10 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
         db = spec ? db : nx.w;
         cq = spec ? cq : nq;
         hi ^= both;
-        full = true;
+        full = moved = true;
         e += n + 1u;
       }
-      if (full) {
+      if (moved) {
         up = hi == 1u << f_hi;
         p.e = e;
         p.Xq = X;
@@ -520,10 +523,12 @@ __device__ __forceinline__ int trace_film(Particle<float>& p, const GeoRun& g, c
         p.d_rel = p.lam * f.E;
       }
       aim();
+      full = false;
     } else {
       p.Xq += cq;
       p.d_rel = p.d_rel - seg;
       p.x[W] = up ? LW : 0.0f;
+      full = true;
       if (up ? iso_hi : iso_lo) return STEP_ABSORBED;
       if (si < nslots) {
         const bool spec = ((d->spec >> (up ? f_hi : f_lo)) & 1u) != 0u;
