@@ -6,9 +6,9 @@
 // from event to event, and the event itself holds the geometry only.  Every
 // value is the event step's own (step_steady, apply_event) bit for bit.
 // Cycles per event of a lone particle (gray, 1 mm free path; 2.07 GHz), before
-// and now: 10 nm film 520 -> 194 (half specular walls 520 -> 208), pore lattice
-// 771 -> 451, its measure-valued gradient 1472 -> 841 and likelihood-ratio
-// gradient 1017 -> 483, square-pore mesh 1379 -> 767.
+// and now: 10 nm film 518 -> 197 (half specular walls 518 -> 198, specular 501 ->
+// 200), pore lattice 771 -> 452, its measure-valued gradient 1470 -> 828 and
+// likelihood-ratio gradient 999 -> 470, square-pore mesh 1374 -> 767.
 #pragma once
 
 #include "tracer.cuh"
